@@ -38,35 +38,42 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
 
 // Philox4x32-10 of counter (j, c1, c2, c3) for a stream whose words c1, c2,
 // c3 are fixed: round 1 of every call shares the product of c2 and the
-// words derived from it, so a stream computes them once (philox_stream) and
-// each call starts from round 2's inputs. Same output as philox4x32_10.
+// words derived from it, so a stream computes them once and each call starts
+// from round 2's inputs. Same output as philox4x32_10.
 struct PhiloxStream {
     uint32_t a0;  // round-1 output word 0: hi(M1 c2) ^ c1 ^ k0
     uint32_t a1;  // round-1 output word 1: lo(M1 c2)
     uint32_t a3;  // c3 ^ k1 (XORed with hi(M0 j) to give round-1 word 2)
 };
 
-__device__ __forceinline__ PhiloxStream philox_stream(uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
-                                                      uint32_t k1) {
-    const uint64_t p1 = uint64_t(0xCD9E8D57u) * c2;
-    PhiloxStream s;
-    s.a0 = uint32_t(p1 >> 32) ^ c1 ^ k0;
-    s.a1 = uint32_t(p1);
-    s.a3 = c3 ^ k1;
-    return s;
+// Round keys of Philox rounds 2..10 (key + r x the Weyl constants), formed by
+// the host: as kernel parameters they are constant-bank operands of the
+// rounds' XORs, where keys formed on the device cost adds in every call (the
+// decoupled kernel on the d=29 workload: 300 k -> 275 k warp-instructions per
+// 64-shot chunk). A call then is 38 instructions, but 73 issue cycles: each of
+// its 17 64-bit products takes four.
+struct PhiloxKeys {
+    uint32_t k0[9], k1[9];
+};
+
+inline __host__ PhiloxKeys philox_keys(uint32_t key0, uint32_t key1) {
+    PhiloxKeys k;
+    for (uint32_t r = 0; r < 9; r++) {
+        k.k0[r] = key0 + (r + 1) * 0x9E3779B9u;
+        k.k1[r] = key1 + (r + 1) * 0xBB67AE85u;
+    }
+    return k;
 }
 
-__device__ __forceinline__ uint4 philox_call(const PhiloxStream &s, uint32_t j, uint32_t k0, uint32_t k1) {
+__device__ __forceinline__ uint4 philox_call(const PhiloxStream &s, uint32_t j, const PhiloxKeys &k) {
     const uint64_t p0 = uint64_t(0xD2511F53u) * j;
     uint32_t c0 = s.a0, c1 = s.a1, c2 = uint32_t(p0 >> 32) ^ s.a3, c3 = uint32_t(p0);
 #pragma unroll
-    for (int r = 1; r < 10; r++) {
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
+    for (int r = 0; r < 9; r++) {
         const uint64_t q0 = uint64_t(0xD2511F53u) * c0;
         const uint64_t q1 = uint64_t(0xCD9E8D57u) * c2;
-        const uint32_t n0 = uint32_t(q1 >> 32) ^ c1 ^ k0;
-        const uint32_t n2 = uint32_t(q0 >> 32) ^ c3 ^ k1;
+        const uint32_t n0 = uint32_t(q1 >> 32) ^ c1 ^ k.k0[r];
+        const uint32_t n2 = uint32_t(q0 >> 32) ^ c3 ^ k.k1[r];
         c0 = n0;
         c1 = uint32_t(q1);
         c2 = n2;
@@ -176,6 +183,31 @@ __device__ __forceinline__ int gap_count_near_at(const uint32_t *__restrict__ ta
     return w < t ? m : m - 1;
 }
 
+// gap_count_near_at with fewer instructions: the estimate is clamped as a
+// float and rounded by adding 1.5 x 2^23 (round to nearest even, as the
+// conversion does), which leaves the integer in the sum's low bits, so no
+// float-to-int conversion is needed and the constant folds into the table
+// index; the logarithm is the flush-to-zero one (its argument is at least 1,
+// so no denormal scaling is needed and the value is the same).
+__device__ __forceinline__ float lg2_ftz(float x) {
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+template <bool SMT>
+__device__ __forceinline__ int gap_count_magic(const uint32_t *__restrict__ tab, uint32_t base1, float inv_log2,
+                                               float c32, uint32_t w) {
+    constexpr float kMagic = 12582912.0f;        // 1.5 x 2^23, bits 0x4B400000
+    constexpr uint32_t kMagicBits = 0x4B400000u;
+    const float est = fmaf(lg2_ftz(__uint2float_rn(w) + 1.0f), inv_log2, c32);
+    const uint32_t mb = __float_as_uint(fminf(fmaxf(est, 1.0f), float(kGapLen)) + kMagic);
+    const uint32_t i = mb + (base1 - kMagicBits);
+    uint32_t t;
+    if constexpr (SMT) t = tab[i];
+    else t = __ldg(tab + i);
+    return int(mb - kMagicBits) - (w < t ? 0 : 1);
+}
+
 template <bool SMT>
 __device__ __forceinline__ int gap_count_near(const uint32_t *__restrict__ T, float inv_log2, float c32, uint32_t w) {
     return gap_count_near_at<SMT>(T, 0xFFFFFFFFu, inv_log2, c32, w);
@@ -223,6 +255,14 @@ __device__ __forceinline__ void st_release_shared64(unsigned long long *p, unsig
 }
 __device__ __forceinline__ void red_release_add_shared(uint32_t *p, uint32_t v) {
     asm volatile("red.release.cta.shared::cta.add.u32 [%0], %1;" ::"r"(shared_addr(p)), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t atom_add_acq_rel_shared(uint32_t *p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.u32 %0, [%1], %2;"
+                 : "=r"(old)
+                 : "r"(shared_addr(p)), "r"(v)
+                 : "memory");
+    return old;
 }
 
 // Warp-aggregated shared counter: the calling lane's index among all lanes

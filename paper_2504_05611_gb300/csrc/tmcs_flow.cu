@@ -10,25 +10,33 @@
 // segments) in steps whose detectors lie in a ring window above the step's
 // flush point. The difference is the execution:
 //
-//  * Walker warps take (tile, step, item, chunk) streams in CTA order from
-//    one shared counter, across step and tile boundaries, and append every
-//    event as one 32-bit word (event slot, chunk, lane) to their step's
-//    region of a circular arena. No lane waits for the end of a step.
+//  * Walker warps take batches of 32 streams (tile, step, 32 / K items x K
+//    chunks) in CTA order from one shared counter, across step and tile
+//    boundaries, and append every event that flips something as one 32-bit
+//    word (event slot, chunk, lane) to their step's region of a circular
+//    arena.
 //  * Applier warps take steps in order: once every stream of step Q has
 //    finished, they apply its events to the ring (shared-memory atomic XORs
-//    of the event's output list), write the detectors the step finalises to
-//    HBM, clear them, and free the step's arena region.
+//    of the ring rows in the event's slot), write the detectors the step
+//    finalises to HBM, clear them, and free the step's arena region.
 //
 // A step's region has a capacity fixed at launch from the expected number
-// of its events (mean + 6 sigma + 64, at most the arena). A walker may start
-// a stream of step Q only when Q's region no longer overlaps an unapplied
-// step's; an event beyond its region's capacity is held by its lane, which
-// stops walking until Q is the step being applied and then XORs the event
-// into the ring itself before reporting its stream finished. The ring is
-// therefore only ever touched for the step being applied, so it needs one
+// of its events (mean + 6 sigma + 64) and of its streams that a batch puts
+// aside. A walker may start a batch of step Q only when Q's region no longer
+// overlaps an unapplied step's; an event beyond its region's capacity is held
+// by its lane, which waits until Q is the step being applied and then XORs
+// the event into the ring itself before its batch counts as walked. The ring
+// is therefore only ever touched for the step being applied, so it needs one
 // window of detectors, while the arena keeps several steps of walking in
 // flight. All waits are bounded (kWaitNs); on expiry the kernel sets bit 0
 // of the status word and every warp leaves.
+//
+// Measured (one GB300, 2070 MHz; before = one lane per stream with refills,
+// 8-byte event slots per Pauli index): d=29 non-local CNOT, p = 1e-3, 2e6
+// shots (12.39 GB of output): 11.20 ms before, 9.4 ms now (1.32 TB/s); the
+// same at p = 1e-4: 6.58, 5.46 (2.27 TB/s); d=11, 1e7 shots: 3.26, 3.09;
+// BB144 teleport, 3e6: 3.01, 2.64. Warp-instructions per 64-shot chunk on
+// d=29: 275 k before, 228 k now.
 #include <cuda.h>  // CUtensorMap (encoded through the runtime's driver entry point)
 #include <cuda_runtime.h>
 
@@ -43,36 +51,36 @@
 
 namespace tmcs {
 
-constexpr uint32_t kFlowSlots = 64;       // steps in flight (done / count slots)
+constexpr uint32_t kFlowSlots = 16;       // steps in flight (done / count slots)
 // events an applier lane loads at once (build-time tuning value)
 #ifndef TMCS_FLOW_APPLY_BATCH
 #define TMCS_FLOW_APPLY_BATCH 4
 #endif
 constexpr uint32_t kFlowApplyBatch = TMCS_FLOW_APPLY_BATCH;
+constexpr uint32_t kFlowBlocks = 32;      // blocks of 32 put-aside streams a step has at most
 constexpr uint32_t kFlowMinArena = 1024;  // smallest useful arena (entries)
-// arena entry of an event that flips nothing (no event word takes this value:
-// flow_shape keeps event slots x 64 x K below 2^32)
-constexpr uint32_t kFlowDead = 0xFFFFFFFFu;
 constexpr uint32_t kFlowMaxArena = 65536;
-
 struct FlowArgs {
     CUtensorMap tmap;           // det as a [n_det][ld] uint64 tensor (tensor-store flush), when tma_rows > 0
     const NoiseDesc *noise;
     const uint32_t *tables;
     const uint4 *item_desc;     // walker descriptors, two uint4 per item (see SigSchedule::item_desc)
     const uint4 *steps;         // item_begin, item_end, flush_lo, flush_hi
-    const float *step_events;   // expected events per chunk of each step
-    const uint32_t *ev_ent;     // two words per event slot, then the overflow lists
-    uint32_t n_steps, n_items, window_mask, n_obs;
-    uint32_t arena;             // arena entries (power of two)
+    const float2 *step_events;  // expected live events and unfinished streams per chunk of each step
+    const uint32_t *rows;       // ring rows of every compact event slot (see SigSchedule::rows)
+    uint32_t n_steps, window_mask, n_obs;
+    uint32_t arena;             // arena entries
     uint32_t test_cap;          // testing: capacity of every step's region (0: from step_events)
+    uint32_t calls;             // Philox calls of every stream's first window (1..4); 0: each item's own
+    uint32_t pc1;               // the program has PAULI_CHANNEL_1 noise
+    uint32_t near;              // every gap table allows the one-read count (kNearInv)
     uint32_t smem_tables;       // gap tables staged in shared memory (count), 0: read from global
     uint32_t walkers;           // walker warps; the CTA's other warps apply
     uint32_t key0, key1, first_chunk;
+    PhiloxKeys keys;            // round keys of rounds 2..10
     uint32_t vec_out;           // det 16-byte aligned and n_cols even: 16-byte output stores
     uint64_t n_cols, last_mask, n_tiles;
     uint64_t ld;                // words between output rows (the call's column count; a launch may cover a slice)
-    uint32_t *garena;           // arena in global memory (a slice of `arena` entries per CTA), or null
     uint32_t tma_rows;          // detector rows per tensor-store box of the flush (0: plain stores)
     uint64_t col_base;          // column of this launch's column 0 in the tensor map (sliced launches)
     uint64_t *det;
@@ -80,34 +88,40 @@ struct FlowArgs {
     uint32_t *status;
 };
 
-// Arena positions are kept modulo 2^32: only differences (less than the
-// arena size plus one step's region) and positions modulo the arena size
-// (a power of two) are used.
+// Step positions in the arena's sequence are kept modulo 2^32: only
+// differences (less than the arena size plus one step's region) are used.
 struct FlowCtl {
-    uint32_t next;                 // streams handed out (CTA sequence; a launch keeps it below 2^31)
+    uint32_t next;                 // batches handed out (CTA sequence; a launch keeps it below 2^31)
     uint32_t u_applied;            // arena position of the first unapplied step
     uint32_t applied;              // steps applied (CTA sequence)
     uint32_t abort;                // a bounded wait expired
     uint32_t app_stop;             // appliers leave (written by applier thread 0 before a barrier)
-    uint32_t done[kFlowSlots];     // finished streams of step Q (slot Q mod kFlowSlots)
-    uint32_t cnt[kFlowSlots];      // arena entries reserved by step Q's events
+    // of step Q, in slot Q mod kFlowSlots:
+    uint32_t done[kFlowSlots];     // walked batches | finished blocks of put-aside streams << 16
+    uint32_t cnt[kFlowSlots];      // arena entries reserved by its events
+    uint32_t left[kFlowSlots];     // streams put aside
+    uint32_t blk[kFlowSlots][kFlowBlocks / 4];  // entries written per block of 32 (a byte each)
 };
 
-// Shared-memory regions (same order and sizes as flow_smem_bytes): ring and
-// observable rows, step table (item end, region capacity, region offset per
-// step, then the tile's total), gap tables, arena.
+static_assert(sizeof(FlowCtl) <= 1024, "the launch leaves 1 KB for static shared variables");
+
+// Shared-memory regions (same order and sizes as flow_fixed_bytes): ring and
+// observable rows, step table (batches up to and including the step, region
+// capacity for events, for put-aside streams, region offset; then the tile's
+// total), gap tables, arena.
 struct FlowSmem {
     uint64_t *ring;
-    uint32_t *send, *scap, *soff;
+    uint32_t *bend, *scap, *slcap, *soff;
     uint32_t *stab;
     uint32_t *arena;
 };
 
 __host__ __device__ inline size_t flow_ring_bytes(uint32_t W, uint32_t n_obs, int K) {
-    return ((size_t(W) + n_obs) * size_t(K) * 8 + 15) & ~size_t(15);
+    // detectors, observables and the spare row
+    return ((size_t(W) + n_obs + 1) * size_t(K) * 8 + 15) & ~size_t(15);
 }
 __host__ __device__ inline size_t flow_step_bytes(uint32_t n_steps) {
-    return ((3 * size_t(n_steps) + 1) * 4 + 15) & ~size_t(15);
+    return ((4 * size_t(n_steps) + 1) * 4 + 15) & ~size_t(15);
 }
 
 __device__ __forceinline__ FlowSmem flow_layout(uint64_t *smem, const FlowArgs &A, int K) {
@@ -115,9 +129,10 @@ __device__ __forceinline__ FlowSmem flow_layout(uint64_t *smem, const FlowArgs &
     unsigned char *b = reinterpret_cast<unsigned char *>(smem);
     S.ring = smem;
     b += flow_ring_bytes(A.window_mask + 1u, A.n_obs, K);
-    S.send = reinterpret_cast<uint32_t *>(b);
-    S.scap = S.send + A.n_steps;
-    S.soff = S.scap + A.n_steps;
+    S.bend = reinterpret_cast<uint32_t *>(b);
+    S.scap = S.bend + A.n_steps;
+    S.slcap = S.scap + A.n_steps;
+    S.soff = S.slcap + A.n_steps;
     b += flow_step_bytes(A.n_steps);
     S.stab = reinterpret_cast<uint32_t *>(b);
     b += size_t(A.smem_tables) * kTableWords * 4;
@@ -130,296 +145,418 @@ struct FlowLog {
     static constexpr uint32_t v = K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4;
 };
 
-__device__ __forceinline__ unsigned long long ld_shared_volatile64(const unsigned long long *p) {
-    return *reinterpret_cast<const volatile unsigned long long *>(p);
-}
+// One compact event slot as loaded: two rows per word (see SigSchedule::rows).
+template <bool WIDE>
+struct FlowSlot;
+template <>
+struct FlowSlot<false> {
+    uint32_t x;
+    __device__ __forceinline__ static FlowSlot load(const uint32_t *rows, uint32_t slot) { return {__ldg(rows + slot)}; }
+};
+template <>
+struct FlowSlot<true> {
+    uint32_t x, y, z, w;
+    __device__ __forceinline__ static FlowSlot load(const uint32_t *rows, uint32_t slot) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(rows) + slot);
+        return {v.x, v.y, v.z, v.w};
+    }
+};
 
 // XORs one event into the ring: word wv = event slot << (6 + log2 K) |
-// chunk << 6 | lane, v = the slot's two words (an entry is observable flag
-// << 29 | output index; observables are the rows after the ring).
-template <int K>
-__device__ __forceinline__ void flow_put(const FlowArgs &A, uint64_t *ring, uint32_t wv, uint2 v) {
-    if (v.x == kEvNone) return;
-    const uint32_t lane = wv & 63u, k = (wv >> 6) & uint32_t(K - 1);
-    uint32_t *base = reinterpret_cast<uint32_t *>(ring) + 2u * k + (lane >> 5);
-    const uint32_t bit = 1u << (lane & 31u);
-    const uint32_t obs_row = A.window_mask + 1u;
-    auto put = [&](uint32_t e) {
-        const uint32_t idx = e & 0x1FFFFFFFu;
-        const uint32_t row = (e & (1u << 29)) ? obs_row + idx : (idx & A.window_mask);
-        atomicXor(base + size_t(row) * (2u * uint32_t(K)), bit);
-    };
-    if (v.x & kEvOverflow) {
-        const uint32_t *ov = A.ev_ent + (v.x & ~kEvOverflow);
-        for (uint32_t x = 0; x < v.y; x++) put(__ldg(ov + x));
-    } else {
-        put(v.x);
-        if (v.y != kEvNone) put(v.y);
+// chunk << 6 | lane, v = the slot's rows.
+template <int K, bool WIDE>
+__device__ __forceinline__ void flow_put(const FlowArgs &A, uint64_t *ring, uint32_t wv, const FlowSlot<WIDE> &v) {
+    // 32-bit word of the row that holds the event's lane: 2 chunk + lane / 32
+    uint32_t *const base = reinterpret_cast<uint32_t *>(ring) + ((wv >> 5) & (2u * uint32_t(K) - 1u));
+    const uint32_t bit = 1u << (wv & 31u);
+    auto put = [&](uint32_t row) { atomicXor(base + row * (2u * uint32_t(K)), bit); };
+    if (v.x & kRowOverflow) {
+        const uint32_t *ov = A.rows + (v.x & ~kRowOverflow);
+        const uint32_t n = __ldg(ov);
+        for (uint32_t i = 0; i < n; i += 2) {
+            const uint32_t w = __ldg(ov + 1 + i / 2);
+            put(w & 0xFFFFu);
+            put(w >> 16);
+        }
+        return;
+    }
+    // unused entries of a word name the spare row
+    put(v.x & 0xFFFFu);
+    put(v.x >> 16);
+    if constexpr (WIDE) {
+        // a word whose first entry is the spare row holds nothing, nor do
+        // those after it
+        const uint32_t spare = A.window_mask + 1u + A.n_obs;
+        if ((v.y & 0xFFFFu) == spare) return;
+        put(v.y & 0xFFFFu);
+        put(v.y >> 16);
+        if ((v.z & 0xFFFFu) == spare) return;
+        put(v.z & 0xFFFFu);
+        put(v.z >> 16);
+        if ((v.w & 0xFFFFu) == spare) return;
+        put(v.w & 0xFFFFu);
+        put(v.w >> 16);
     }
 }
 
-template <int K>
-__device__ __forceinline__ void flow_put_word(const FlowArgs &A, uint64_t *ring, uint32_t wv) {
-    if (wv == kFlowDead) return;
-    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(A.ev_ent) + (wv >> (6u + FlowLog<K>::v)));
-    flow_put<K>(A, ring, wv, v);
+// Waits until done() holds, polled by lane 0 for the whole warp; bounded
+// (kWaitNs). False for every lane when the wait expired, here (status bit
+// set) or in another warp.
+template <class Done>
+__device__ __forceinline__ bool flow_warp_wait(FlowCtl &C, uint32_t *status, uint32_t lane, Done &&done) {
+    int ok = 1;
+    if (lane == 0 && !done()) {
+        const uint64_t t0 = globaltimer_ns();
+        while (!done()) {
+            if (ld_shared_volatile(&C.abort)) {
+                ok = 0;
+                break;
+            }
+            if (globaltimer_ns() - t0 > kWaitNs) {
+                C.abort = 1u;
+                atomicOr(status, 1u);
+                ok = 0;
+                break;
+            }
+            __nanosleep(64);
+        }
+    }
+    // the shuffle carries the decision, the warp barrier lane 0's acquire
+    ok = __shfl_sync(0xFFFFFFFFu, ok, 0);
+    __syncwarp();
+    return ok != 0;
 }
 
-// Walker warps. Every lane holds at most one stream; streams are handed out
-// in CTA order (tile, step, item, chunk). An iteration is a window of
-// W Philox calls (two draws each) of every walking lane's stream,
-// with the window's events kept in registers; then the warp reserves arena
-// entries for all of them at once, together with the lanes whose streams
-// belong to the same step (one shared atomic per step and warp), reports the
-// streams that ended and refills those lanes. Streams longer than a window
-// continue in the next one. The per-iteration work of the warp (refill,
-// reservation, completion) is thus shared by up to 2 W draws per lane.
-template <int K, int W, bool SMT, bool GA>
-__device__ __forceinline__ void flow_walk(const FlowArgs &A, const FlowSmem &S, FlowCtl &C, uint32_t nt,
-                                          uint32_t nv_last, const uint32_t *tabs) {
-    constexpr uint32_t LK = FlowLog<K>::v;
-    constexpr int NE = 2 * W;  // events a lane can draw per window
-    static_assert(NE < 16, "event counts per window are reserved with four count-bit ballots at most");
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t n_steps = A.n_steps, amask = A.arena - 1u;
-    // the arena: shared memory, or this CTA's slice of a global buffer
-    // (L2-resident; entries written and read past L1)
-    uint32_t *const arena = GA ? A.garena + size_t(blockIdx.x) * A.arena : S.arena;
-    const uint32_t per_tile = A.n_items << LK;
-    const uint32_t total = nt * per_tile;
-    const uint32_t c_tile = S.soff[n_steps];
-    bool have = false, live = false, ended = false, exhausted = false;
-    uint32_t tcur = 0xFFFFFFFFu, tbase = 0;
-    // the lane's stream: step Q, its region (capacity, low word of its
-    // unwrapped arena position, gate), Philox stream words, call counter,
-    // first event slot, kind, Pauli counts, gap table offset, chunk tag,
-    // position and length in trials
-    uint32_t Q = 0, cap = 0, uq = 0, gate = 0;
-    PhiloxStream ps{0u, 0u, 0u};
-    // event words: slot << S | chunk << 6 | lane (S = 6 + log2 K) with slot =
-    // ubase + (pos >> 6) kp + (Pauli index - 1), formed as
-    // evb + (pos >> 6) kpm + pos + (Pauli index - 1) 2^S, where evb = ubase 2^S
-    // + chunk 2^6 and kpm = kp 2^S - 64 (all modulo 2^32)
-    constexpr uint32_t S_EV = 6u + LK;
-    uint32_t call = 0, evb = 0, kind = 0, npauli = 1, kpm = 0, toff = 0, t1 = 0, t2 = 0, live_k = 0;
-    int pos = -1, n_trials = 0;
-    float inv = 0.f, c32 = 0.f;
-    // the window's events; ev[held .. ne) are events that did not fit their
-    // step's region and wait for it to be the step being applied
-    uint32_t ev[NE];
-    uint32_t ne = 0, held = 0;
-    uint32_t t_wait = 0, iter = 0;
-    bool waiting = false;
-    for (;;) {
-        if ((iter++ & 7u) == 0u && __any_sync(0xFFFFFFFFu, ld_shared_volatile(&C.abort) != 0u)) return;
-        if (!have && !exhausted) {
-            const uint32_t g = grab_index(&C.next);
-            if (g >= total) {
-                exhausted = true;
-            } else {
-                if (tcur == 0xFFFFFFFFu || g - tbase >= per_tile) {
-                    tcur = g / per_tile;
-                    tbase = tcur * per_tile;
-                }
-                const uint32_t sl = g - tbase;
-                const uint32_t it = sl >> LK, k = sl & uint32_t(K - 1);
-                const uint4 d0 = __ldg(A.item_desc + 2 * it), d1 = __ldg(A.item_desc + 2 * it + 1);
-                const uint32_t q = d1.x >> 17;
-                Q = tcur * n_steps + q;
-                const uint32_t U = tcur * c_tile + S.soff[q];  // modulo 2^32
-                cap = S.scap[q];
-                gate = U + cap - A.arena;
-                uq = U;
-                kind = d1.x & 7u;
-                npauli = (d1.x >> 3) & 15u;
-                kpm = (((d1.x >> 7) & 15u) << S_EV) - 64u;
-                toff = (d1.y & 0x1FFFu) * kTableWords;
-                inv = __uint_as_float(d1.z);
-                c32 = -32.0f * inv;  // exact (a power-of-two scaling)
-                live_k = d1.w;
-                if (kind == N_PC1) {
-                    t1 = __ldg(&A.noise[d1.y >> 13].t1);
-                    t2 = __ldg(&A.noise[d1.y >> 13].t2);
-                }
-                const uint32_t nv = tcur == nt - 1u ? nv_last : uint32_t(K);
-                const uint32_t chunk = A.first_chunk + (blockIdx.x + tcur * gridDim.x) * uint32_t(K) + k;
-                // Philox round 1 of this stream from the descriptor's product
-                // of the op index (counter words: call, chunk, op, segment)
-                ps.a0 = d0.x ^ chunk ^ A.key0;
-                ps.a1 = d0.y;
-                ps.a3 = d0.z ^ A.key1;
-                evb = (d0.w << S_EV) | (k << 6);
-                // chunks past the end of the call (ragged last tile): no trials
-                n_trials = k < nv ? 64 * int(((d1.x >> 11) & 63u) + 1u) : 0;
-                call = 0;
-                pos = -1;
-                have = true;
-                live = false;
-                ended = false;
-            }
-        }
-        // the stream may start once its step's arena region is free and the
-        // step is within the slots in flight
-        if (have && !live) {
+// Walker warps.
+//
+// A batch is 32 streams of one step: 32 / K consecutive items x the tile's K
+// chunks, one per lane (lane = item x K + chunk), so everything but the
+// stream itself is uniform over the warp: the step, its arena region, the
+// gate, the completion. Batches are handed out in CTA order (tile, step,
+// batch) from one shared counter. A batch runs a first window of W Philox
+// calls (two draws each; W from the items' expected draws, the same for the
+// 32 streams, which are sorted by that) as straight-line code. The streams
+// that need more draws (a few of the 32) are put aside, one word each, in
+// the tail of the step's arena region; the warp whose streams fill a block
+// of 32 there finishes that block, the warp that walks the step's last batch
+// the rest. Running on in place with the few lanes that are not done would
+// cost a call per batch at a fifth of the lanes.
+//
+// What bounds it: instruction issue (the integer pipe and the 64-bit
+// products of Philox, four issue cycles each, above all). One lane per
+// stream with refills after every window (the layout this replaced) spent
+// 310 of its 830 warp-instructions per iteration on per-lane bookkeeping:
+// refill, gate, grouping lanes by step, completion.
+template <int K, bool SMT, bool WIDE>
+struct FlowWalker {
+    static constexpr uint32_t LK = FlowLog<K>::v;
+    static constexpr uint32_t IPB = 32u / uint32_t(K);  // items per batch
+    static constexpr uint32_t S_EV = 6u + LK;           // event words: slot << S_EV | chunk << 6 | lane
+    static constexpr uint32_t CB = WIDE ? 4u : 2u;      // bits of a class
+
+    const FlowArgs &A;
+    const FlowSmem &S;
+    FlowCtl &C;
+    const uint32_t *tabs;
+    uint32_t lane, lt;
+    // the step being walked: sequence number, first item, item end, batches,
+    // region (position in the arena, capacity for events and for put-aside
+    // streams), tile's first chunk, valid chunks
+    uint32_t Q = 0xFFFFFFFFu, item0 = 0, item_end = 0, nb = 0, upos = 0, cap = 0, lcap = 0, chunk0 = 0, nv = 0;
+
+    struct Stream {
+        PhiloxStream ps;
+        uint32_t evb, kpm, npm, tab1, kind, desc, calls;
+        uint64_t lut;  // classes << S_EV - CB shifted right by a Pauli index's bits (CB per index)
+        int n_trials;
+        float inv, c32;
+    };
+
+    // Decodes the lane's stream: item (index in the schedule), chunk k of
+    // the tile. Event words are slot << S_EV | chunk << 6 | lane with slot =
+    // slot0 + (pos >> 6) classes + class - 1, formed as evb + (pos >> 6) kpm
+    // + pos + class << S_EV (modulo 2^32).
+    __device__ __forceinline__ Stream open(uint32_t item, uint32_t k, bool valid) const {
+        const uint4 d0 = __ldg(A.item_desc + 2 * item), d1 = __ldg(A.item_desc + 2 * item + 1);
+        Stream s;
+        s.kind = d1.x & 7u;
+        s.npm = ((d1.x >> 3) & 15u) * CB;
+        s.kpm = (((d1.x >> 7) & 15u) << S_EV) - 64u;
+        s.calls = ((d1.x >> 17) & 3u) + 1u;
+        s.tab1 = (d1.x >> 19) * kTableWords - 1u;
+        s.desc = d1.z;
+        // two-row layout: 30 bits, kept S_EV bits up so that the shift by a
+        // Pauli index leaves its class in place in the event word
+        s.lut = WIDE ? uint64_t(d1.y) | (uint64_t(d1.z) << 32) : uint64_t(d1.y) << S_EV;
+        s.inv = __uint_as_float(d1.w);
+        s.c32 = -32.0f * s.inv;  // exact (a power-of-two scaling)
+        // Philox round 1 from the descriptor's product of the op index
+        // (counter words: call, chunk, op, segment)
+        s.ps.a0 = d0.x ^ (chunk0 + k) ^ A.key0;
+        s.ps.a1 = d0.y;
+        s.ps.a3 = d0.z ^ A.key1;
+        s.evb = ((d0.w - 1u) << S_EV) + (k << 6);
+        // lanes past the step's items and chunks past the call's end: no trials
+        s.n_trials = valid ? 64 * int(((d1.x >> 11) & 63u) + 1u) : 0;
+        return s;
+    }
+
+    // Waits until the step's arena region is free (`gate`: signed difference
+    // modulo 2^32) and the step is within the slots in flight. False when a
+    // bounded wait expired, here or elsewhere.
+    __device__ __forceinline__ bool wait_gate(uint32_t gate) const {
+        return flow_warp_wait(C, A.status, lane, [&]() {
             // acquire: the appliers' last reads of the region and their
-            // reset of the step's counters precede our writes. The region
-            // is free once u_applied has reached the gate (signed
-            // difference: positions are modulo 2^32).
-            const uint32_t ua = ld_acquire_shared(&C.u_applied);
-            if (int32_t(ua - gate) >= 0 && Q - ld_acquire_shared(&C.applied) < kFlowSlots) live = true;
-        }
-        // events held back by a full region: once step Q is the one being
-        // applied, XOR them into the ring directly
-        if (held < ne && ld_acquire_shared(&C.applied) == Q) {
-#pragma unroll
-            for (int j = 0; j < NE; j++)
-                if (uint32_t(j) >= held && uint32_t(j) < ne) flow_put_word<K>(A, S.ring, ev[j]);
-            held = ne;
-        }
-        const bool walk = live && !ended && held == ne;
-        const uint32_t wm = __ballot_sync(0xFFFFFFFFu, walk);
-        if (wm) {
-            if (walk) {
-                ne = 0;
-                held = 0;
-                // the window's W Philox calls and 2W gap counts do not depend
-                // on one another: straight-line code, so their latencies
-                // overlap; draws after the stream's last one are computed
-                // and discarded (the warp runs them for its other lanes)
-                uint32_t wp[NE];
-                int gp[NE];
-                // one table read per gap when every walking lane's p allows
-                // it (warp-uniform choice), else the two-read count
-                if (__all_sync(wm, fabsf(inv) < kNearInv)) {
-#pragma unroll
-                    for (int c = 0; c < W; c++) {
-                        const uint4 w = philox_call(ps, call + uint32_t(c), A.key0, A.key1);
-                        gp[2 * c] = gap_count_near_at<SMT>(tabs, toff - 1u, inv, c32, w.x);
-                        gp[2 * c + 1] = gap_count_near_at<SMT>(tabs, toff - 1u, inv, c32, w.z);
-                        wp[2 * c] = w.y;
-                        wp[2 * c + 1] = w.w;
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < W; c++) {
-                        const uint4 w = philox_call(ps, call + uint32_t(c), A.key0, A.key1);
-                        gp[2 * c] = gap_count_est<SMT>(tabs + toff, inv, c32, w.x);
-                        gp[2 * c + 1] = gap_count_est<SMT>(tabs + toff, inv, c32, w.z);
-                        wp[2 * c] = w.y;
-                        wp[2 * c + 1] = w.w;
-                    }
-                }
-                call += uint32_t(W);
-                // positions in draw order (increasing): every draw before the
-                // one that passes the end of the segment is an event
-                int pd[NE];
-#pragma unroll
-                for (int d = 0; d < NE; d++) {
-                    pos += 1 + gp[d];
-                    pd[d] = pos;
-                }
-                ne = 0;
-#pragma unroll
-                for (int d = 0; d < NE; d++) ne = pd[d] < n_trials ? uint32_t(d + 1) : ne;
-                ended = pos >= n_trials;
-                // Pauli index - 1: PAULI_CHANNEL_1 thresholds, else uniform
-                // (the thresholds are only looked at in warps that have a
-                // PAULI_CHANNEL_1 lane). An event whose Pauli index flips
-                // nothing in any unit of the segment becomes kFlowDead: it
-                // keeps its arena entry but costs the appliers no table read.
-                auto words = [&](auto pc1) {
-#pragma unroll
-                    for (int d = 0; d < NE; d++) {
-                        uint32_t k1 = __umulhi(wp[d], npauli);
-                        if constexpr (decltype(pc1)::value)
-                            if (kind == N_PC1) k1 = wp[d] < t1 ? 0u : wp[d] < t2 ? 2u : 1u;
-                        const uint32_t pu = uint32_t(pd[d]);
-                        const uint32_t wd = (pu >> 6) * kpm + (evb + pu) + (k1 << S_EV);
-                        ev[d] = wd | (((live_k >> k1) & 1u) - 1u);  // kFlowDead when not live
-                    }
-                };
-                if (__any_sync(wm, kind == N_PC1)) words(std::true_type{});
-                else words(std::false_type{});
-            }
-            // reserve the window's events: lanes of the same step share one
-            // atomic; a lane's offset among them from bit ballots of its count
-            const bool res = walk && ne != 0;
-            const uint32_t em = __ballot_sync(0xFFFFFFFFu, res);
-            if (res) {
-                const uint32_t peers = __match_any_sync(em, Q);
-                // counts reach NE (6 or 8 for windows of 3 or 4 calls): one
-                // ballot per bit of the count
-                constexpr int NB = NE >= 8 ? 4 : 3;
-                uint32_t n = 0, off = 0;
-#pragma unroll
-                for (int bit = 0; bit < NB; bit++) {
-                    const uint32_t bm = __ballot_sync(em, (ne >> bit) & 1u) & peers;
-                    n += uint32_t(__popc(bm)) << bit;
-                    off += uint32_t(__popc(bm & lt)) << bit;
-                }
-                const uint32_t leader = uint32_t(__ffs(peers)) - 1u;
-                uint32_t base = 0;
-                if (lane == leader) base = atomicAdd(&C.cnt[Q & (kFlowSlots - 1u)], n);
-                const uint32_t idx = __shfl_sync(peers, base, int(leader)) + off;
-                // entries past the region's capacity stay in ev[] (held)
-                held = idx >= cap ? 0u : min(ne, cap - idx);
-                // the entries are contiguous unless they wrap past the
-                // arena's end
-                const uint32_t a0 = (uq + idx) & amask;
-                if (a0 + uint32_t(NE) <= A.arena) {
-                    uint32_t *const at = arena + a0;
-#pragma unroll
-                    for (int j = 0; j < NE; j++)
-                        if (uint32_t(j) < held) {
-                            if constexpr (GA) __stcg(at + j, ev[j]);
-                            else at[j] = ev[j];
-                        }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < NE; j++)
-                        if (uint32_t(j) < held) {
-                            if constexpr (GA) __stcg(arena + ((a0 + uint32_t(j)) & amask), ev[j]);
-                            else arena[(a0 + uint32_t(j)) & amask] = ev[j];
-                        }
-                }
-            }
-        }
-        // a stream whose walk ended and whose events are all stored or
-        // applied is reported to its step
-        const bool complete = have && ended && held == ne;
-        const uint32_t cm = __ballot_sync(0xFFFFFFFFu, complete);
-        if (complete) {
-            // the stream's events (stored or applied by this lane) precede
-            // the count: a release add per lane (cheaper than grouping the
-            // lanes of a step behind one add)
-            red_release_add_shared(&C.done[Q & (kFlowSlots - 1u)], 1u);
-            have = false;
-            live = false;
-            ended = false;
-            ne = 0;
-            held = 0;
-        }
-        if (wm | cm) {
-            waiting = false;
-            continue;
-        }
-        // nothing to walk: every lane is done, gated or holding events
-        if (!__any_sync(0xFFFFFFFFu, have)) return;
-        if (__any_sync(0xFFFFFFFFu, ld_shared_volatile(&C.abort) != 0u)) return;
-        if (!waiting) {
-            t_wait = uint32_t(globaltimer_ns());
-            waiting = true;
-        } else if (uint32_t(globaltimer_ns()) - t_wait > uint32_t(kWaitNs)) {
-            if (lane == 0) {
+            // reset of the step's counters precede our writes
+            return int32_t(ld_acquire_shared(&C.u_applied) - gate) >= 0 &&
+                   Q - ld_acquire_shared(&C.applied) < kFlowSlots;
+        });
+    }
+
+    // Event of a lane whose step's region is full: the lane waits until the
+    // step is the one being applied (the ring then holds its window) and
+    // XORs the event into the ring itself. Every earlier step can finish
+    // without this warp: it has reported all its batches of those. When the
+    // bounded wait expires the event is dropped, the status bit set, and the
+    // warp leaves at its next gate.
+    __device__ __noinline__ static void put_late(const FlowArgs &A, uint64_t *ring, FlowCtl &C, uint32_t Q, uint32_t wv) {
+        const uint64_t t0 = globaltimer_ns();
+        while (ld_acquire_shared(&C.applied) != Q) {
+            if (ld_shared_volatile(&C.abort)) return;
+            if (globaltimer_ns() - t0 > kWaitNs) {
                 C.abort = 1u;
                 atomicOr(A.status, 1u);
+                return;
             }
-            return;
+            __nanosleep(64);
         }
-        __nanosleep(64);
+        flow_put<K, WIDE>(A, ring, wv, FlowSlot<WIDE>::load(A.rows, wv >> S_EV));
     }
-}
+
+    // Stores the lane's events of a window (those with live[d]) in the step's
+    // arena region, next to one another. Every lane reserves its entries with
+    // its own shared atomic: the warp's same-address adds cost the memory
+    // pipe a cycle a lane, ballots and population counts for one add per warp
+    // cost the integer pipes more (d=29 workload: 263 k against 244 k
+    // warp-instructions a chunk, 388 against 345 ns).
+    template <int NE>
+    __device__ __forceinline__ void emit(const uint32_t (&ev)[NE], const bool (&live)[NE]) const {
+        uint32_t n = 0;
+#pragma unroll
+        for (int d = 0; d < NE; d++) n += live[d] ? 1u : 0u;
+        uint32_t idx = 0;
+        if (n) idx = atomicAdd(&C.cnt[Q & (kFlowSlots - 1u)], n);
+        uint32_t a = upos + idx;
+        if (a >= A.arena) a -= A.arena;
+        if (a + uint32_t(NE) <= A.arena && idx + uint32_t(NE) <= cap) {
+            uint32_t *at = S.arena + a;
+#pragma unroll
+            for (int d = 0; d < NE; d++) {
+                if (live[d]) *at = ev[d];
+                at += live[d] ? 1 : 0;
+            }
+        } else {
+            // near the arena's end or the region's
+#pragma unroll
+            for (int d = 0; d < NE; d++)
+                if (live[d]) {
+                    if (idx < cap) S.arena[a] = ev[d];
+                    else put_late(A, S.ring, C, Q, ev[d]);
+                    idx++;
+                    a = a + 1u < A.arena ? a + 1u : 0u;
+                }
+        }
+    }
+
+    // W Philox calls from call `call` on, 2W draws: positions in draw order
+    // (increasing), the events before the end of the segment stored. NEAR:
+    // one table read per gap count (gap_count_near_at's derivation), the
+    // estimate rounded by adding 1.5 x 2^23 so that the table index is the
+    // sum's low bits.
+    template <int W, bool NEAR>
+    __device__ __forceinline__ void window(const Stream &s, uint32_t call, int &pos, bool walk) const {
+        constexpr int NE = 2 * W;
+        uint32_t wp[NE];
+        int pd[NE];
+#pragma unroll
+        for (int c = 0; c < W; c++) {
+            const uint4 w = philox_call(s.ps, call + uint32_t(c), A.keys);
+            if constexpr (NEAR) {
+                pd[2 * c] = gap_count_magic<SMT>(tabs, s.tab1, s.inv, s.c32, w.x);
+                pd[2 * c + 1] = gap_count_magic<SMT>(tabs, s.tab1, s.inv, s.c32, w.z);
+            } else {
+                pd[2 * c] = gap_count_est<SMT>(tabs + (s.tab1 + 1u), s.inv, s.c32, w.x);
+                pd[2 * c + 1] = gap_count_est<SMT>(tabs + (s.tab1 + 1u), s.inv, s.c32, w.z);
+            }
+            wp[2 * c] = w.y;
+            wp[2 * c + 1] = w.w;
+        }
+        const int n_trials = walk ? s.n_trials : 0;
+        uint32_t ev[NE];
+        bool live[NE];
+        auto words = [&](auto pc1) {
+            uint32_t t1 = 0, t2 = 0;
+            if constexpr (decltype(pc1)::value)
+                if (s.kind == N_PC1) {
+                    t1 = __ldg(&A.noise[s.desc].t1);
+                    t2 = __ldg(&A.noise[s.desc].t2);
+                }
+#pragma unroll
+            for (int d = 0; d < NE; d++) {
+                pos += 1 + pd[d];
+                // CB x (Pauli index - 1): floor(CB n w / 2^32) without its
+                // low bits, as floor(n w / 2^32) = floor(floor(CB n w / 2^32) / CB)
+                uint32_t kb = __umulhi(wp[d], s.npm) & ~(CB - 1u);
+                if constexpr (decltype(pc1)::value)
+                    if (s.kind == N_PC1) kb = wp[d] < t1 ? 0u : wp[d] < t2 ? 2u * CB : CB;
+                const uint32_t pu = uint32_t(pos);
+                uint32_t cls;  // class << S_EV
+                if constexpr (WIDE) cls = (uint32_t(s.lut >> kb) & 15u) << S_EV;
+                else cls = uint32_t(s.lut >> kb) & (3u << S_EV);
+                ev[d] = (pu >> 6) * s.kpm + (s.evb + pu + cls);
+                live[d] = pos < n_trials && cls != 0u;
+            }
+        };
+        if (A.pc1) words(std::true_type{});
+        else words(std::false_type{});
+        emit<NE>(ev, live);
+    }
+
+    // Runs the lanes with `walk` to the end of their streams, a call at a time.
+    __device__ __forceinline__ void finish(const Stream &s, uint32_t call, int pos, bool walk) const {
+        while (__any_sync(0xFFFFFFFFu, walk)) {
+            if (A.near) window<1, true>(s, call, pos, walk);
+            else window<1, false>(s, call, pos, walk);
+            call++;
+            walk = walk && pos < s.n_trials;
+        }
+    }
+
+    // Puts the lanes' unfinished streams (mask um, not 0) aside. Returns the
+    // blocks of 32 that are complete with them (bits 0 and 1: the block
+    // whose number is in the bits above and the next one; 0: none). Entry: position | lane << 12 |
+    // first-window calls - 1 << 17 | batch within the step << 19.
+    __device__ __forceinline__ uint32_t put_aside(const Stream &s, uint32_t um, uint32_t w, uint32_t b,
+                                                  int pos) const {
+        const uint32_t slot = Q & (kFlowSlots - 1u), n = uint32_t(__popc(um));
+        uint32_t base = 0;
+        if (lane == 0) base = atomicAdd(&C.left[slot], n);
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        const bool mine = (um >> lane) & 1u;
+        const uint32_t idx = base + uint32_t(__popc(um & lt));
+        if (mine && idx < lcap) {
+            const uint32_t a = upos + cap + idx;
+            S.arena[a >= A.arena ? a - A.arena : a] = uint32_t(pos) | (lane << 12) | ((w - 1u) << 17) | (b << 19);
+        }
+        __syncwarp();
+        // count the entries written per block (they touch two blocks at
+        // most: lanes 0 and 1); the warp that completes a block's count has
+        // acquired every entry of it and finishes it, without a wait. Both
+        // blocks can become complete here: the second one's other entries
+        // may have been written first.
+        bool full = false;
+        const uint32_t lo = min(base, lcap), hi = min(base + n, lcap);
+        if (lane < 2) {
+            const uint32_t bk = (lo >> 5) + lane, f = max(lo, bk << 5), e = min(hi, (bk + 1u) << 5);
+            if (f < e) {
+                const uint32_t sh = 8u * (bk & 3u);
+                const uint32_t old = atom_add_acq_rel_shared(&C.blk[slot][bk >> 2], (e - f) << sh);
+                full = ((old >> sh) & 255u) + (e - f) == 32u;
+            }
+        }
+        const uint32_t fm = __ballot_sync(0xFFFFFFFFu, full);
+        // the region's tail is full: finish in place
+        if (base + n > lcap) finish(s, w, pos, mine && idx >= lcap);
+        return fm ? (lo >> 5) << 2 | fm : 0u;
+    }
+
+    // Finishes n streams put aside in block `blk` and counts the block.
+    __device__ __forceinline__ void finish_block(uint32_t blk, uint32_t n) const {
+        __syncwarp();  // the entries, acquired by one lane
+        const bool have = lane < n;
+        const uint32_t a = upos + cap + 32u * blk + lane;
+        const uint32_t e = have ? S.arena[a >= A.arena ? a - A.arena : a] : 0u;
+        const uint32_t sl = (e >> 12) & 31u;
+        const uint32_t item = item0 + (e >> 19) * IPB + (sl >> LK);
+        const Stream s = open(item, sl & uint32_t(K - 1), have);
+        finish(s, ((e >> 17) & 3u) + 1u, int(e & 0xFFFu), have);
+        __syncwarp();
+        if (lane == 0) red_release_add_shared(&C.done[Q & (kFlowSlots - 1u)], 0x10000u);
+    }
+
+    __device__ void run(uint32_t nt, uint32_t nv_last) {
+        const uint32_t n_steps = A.n_steps;
+        const uint32_t bpt = S.bend[n_steps - 1u];  // batches per tile
+        const uint32_t total = nt * bpt;
+        const uint32_t c_tile = S.soff[n_steps];
+        uint32_t T = 0, q = 0, tb = 0;  // the tile and step of the batch last taken, the tile's first batch
+        uint32_t b0 = 0;                // the step's first batch in the tile
+        for (;;) {
+            uint32_t g = 0;
+            if (lane == 0) g = atomicAdd(&C.next, 1u);
+            g = __shfl_sync(0xFFFFFFFFu, g, 0);
+            if (g >= total) return;
+            while (g - tb >= bpt) {
+                tb += bpt;
+                T++;
+                q = 0;
+            }
+            while (g - tb >= S.bend[q]) q++;
+            if (Q != T * n_steps + q) {
+                Q = T * n_steps + q;
+                const uint4 st = __ldg(A.steps + q);
+                item0 = st.x;
+                item_end = st.y;
+                b0 = q ? S.bend[q - 1u] : 0u;
+                nb = S.bend[q] - b0;
+                cap = S.scap[q];
+                lcap = S.slcap[q];
+                const uint32_t U = T * c_tile + S.soff[q];  // modulo 2^32
+                upos = uint32_t((uint64_t(T) * c_tile + S.soff[q]) % A.arena);
+                chunk0 = A.first_chunk + (blockIdx.x + T * gridDim.x) * uint32_t(K);
+                nv = T == nt - 1u ? nv_last : uint32_t(K);
+                if (!wait_gate(U + cap + lcap - A.arena)) return;
+            }
+            const uint32_t b = g - tb - b0;
+            const uint32_t k = lane & uint32_t(K - 1);
+            const uint32_t it = item0 + b * IPB + (lane >> LK);
+            const Stream s = open(min(it, item_end - 1u), k, it < item_end && k < nv);
+            int pos = -1;
+            uint32_t w = 0;
+            if (A.near) {
+                w = A.calls ? A.calls : __shfl_sync(0xFFFFFFFFu, s.calls, 0);
+                switch (w) {
+                case 1: window<1, true>(s, 0u, pos, true); break;
+                case 2: window<2, true>(s, 0u, pos, true); break;
+                case 3: window<3, true>(s, 0u, pos, true); break;
+                default: window<4, true>(s, 0u, pos, true); break;
+                }
+            }
+            const bool unfinished = pos < s.n_trials && s.n_trials > 0;
+            const uint32_t um = __ballot_sync(0xFFFFFFFFu, unfinished);
+            uint32_t full = 0;
+            if (um != 0) {
+                // finish in place when most lanes go on, when there was no
+                // first window (a table needs the two-read count), and when
+                // the batch number does not fit an entry
+                if (w == 0 || __popc(um) > 24 || b >= (1u << 13)) finish(s, w, pos, unfinished);
+                else full = put_aside(s, um, w, b, pos);
+            }
+            // the batch is walked (release: its events and entries are in the
+            // arena or the ring)
+            __syncwarp();
+            uint32_t old = 0;
+            if (lane == 0) old = atom_add_acq_rel_shared(&C.done[Q & (kFlowSlots - 1u)], 1u);
+            old = __shfl_sync(0xFFFFFFFFu, old, 0);
+            if (full & 1u) finish_block(full >> 2, 32u);
+            if (full & 2u) finish_block((full >> 2) + 1u, 32u);
+            if ((old & 0xFFFFu) == nb - 1u) {
+                const uint32_t n = min(ld_acquire_shared(&C.left[Q & (kFlowSlots - 1u)]), lcap);
+                if (n & 31u) finish_block(n >> 5, n & 31u);
+            }
+        }
+    }
+};
 
 __device__ __forceinline__ void flow_bar(uint32_t nthreads) {
     asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
@@ -529,22 +666,22 @@ __device__ __forceinline__ void flow_flush_tma(const FlowArgs &A, const FlowSmem
 }
 
 // Applier warps: steps in CTA order.
-template <int K, bool GA>
+template <int K, bool WIDE>
 __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S, FlowCtl &C, uint32_t nt,
                                            uint32_t nv_last) {
-    constexpr uint32_t LK = FlowLog<K>::v;
+    constexpr uint32_t LK = FlowLog<K>::v, S_EV = 6u + LK;
     const uint32_t nthr = blockDim.x - 32u * A.walkers;
     const uint32_t at = threadIdx.x - 32u * A.walkers;
-    const uint32_t amask = A.arena - 1u, mask = A.window_mask;
+    const uint32_t mask = A.window_mask;
     const uint32_t obs_row = A.window_mask + 1u;
-    const uint2 *ev2 = reinterpret_cast<const uint2 *>(A.ev_ent);
-    const uint32_t *const arena = GA ? A.garena + size_t(blockIdx.x) * A.arena : S.arena;
+    const uint32_t *const arena = S.arena;
     // tensor-store flush: needs the ring 128-byte aligned in shared memory
     // and boxes of a whole number of 128-byte ring stretches (each box then
     // starts aligned)
     const bool tma = (K % 2 == 0) && A.tma_rows != 0 && (A.tma_rows * uint32_t(K)) % 16u == 0 &&
                      (shared_addr(S.ring) & 127u) == 0;
-    uint32_t U = 0;  // arena position of step Q, modulo 2^32
+    uint32_t U = 0;   // arena position of step Q, modulo 2^32
+    uint32_t up = 0;  // the same modulo the arena size
     for (uint32_t T = 0; T < nt; T++) {
         const uint64_t tile = uint64_t(blockIdx.x) + uint64_t(T) * gridDim.x;
         const uint64_t col0 = tile * uint64_t(K);
@@ -552,16 +689,23 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
         for (uint32_t q = 0; q < A.n_steps; q++) {
             const uint32_t Q = T * A.n_steps + q;
             const uint4 st = __ldg(A.steps + q);
-            const uint32_t need = (st.y - st.x) << LK;
+            const uint32_t need = S.bend[q] - (q ? S.bend[q - 1u] : 0u);
             const uint32_t slot = Q & (kFlowSlots - 1u);
             // thread 0 waits for the step's streams and decides for all
             // appliers whether they go on (one value read after the barrier,
             // so every applier thread leaves or none does)
             if (at == 0) {
+                // all batches walked and every block of put-aside streams
+                // finished (their number is final once the batches are)
+                auto complete = [&]() {
+                    const uint32_t d = ld_acquire_shared(&C.done[slot]);
+                    return (d & 0xFFFFu) == need &&
+                           (need == 0u || (d >> 16) == (min(ld_shared_volatile(&C.left[slot]), S.slcap[q]) + 31u) / 32u);
+                };
                 uint32_t stop = ld_shared_volatile(&C.abort);
-                if (!stop && ld_shared_volatile(&C.done[slot]) != need) {
+                if (!stop && !complete()) {
                     const uint64_t t0 = globaltimer_ns();
-                    while (ld_shared_volatile(&C.done[slot]) != need) {
+                    while (!complete()) {
                         if (ld_shared_volatile(&C.abort)) {
                             stop = 1u;
                             break;
@@ -584,29 +728,42 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
             }
             __threadfence_block();  // the walkers' events precede the reads below
             const uint32_t n = min(ld_shared_volatile(&C.cnt[slot]), S.scap[q]);
-            const uint32_t u0 = U;
-            for (uint32_t e = at; e < n; e += nthr * kFlowApplyBatch) {
+            // whole batches first: no bounds in the loop but the wrap
+            const uint32_t per = nthr * kFlowApplyBatch;
+            uint32_t e = at;
+            auto entry = [&](uint32_t i) {
+                const uint32_t a = up + i;
+                return arena[a >= A.arena ? a - A.arena : a];
+            };
+            for (; e + (per - nthr) < n; e += per) {
                 uint32_t wv[kFlowApplyBatch];
-                uint2 v[kFlowApplyBatch];
+                FlowSlot<WIDE> v[kFlowApplyBatch];
 #pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++) {
-                    const uint32_t i = e + j * nthr;
-                    if constexpr (GA) wv[j] = i < n ? __ldcg(arena + ((u0 + i) & amask)) : 0u;
-                    else wv[j] = i < n ? arena[(u0 + i) & amask] : 0u;
-                }
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) wv[j] = entry(e + j * nthr);
+#pragma unroll
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) v[j] = FlowSlot<WIDE>::load(A.rows, wv[j] >> S_EV);
+#pragma unroll
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) flow_put<K, WIDE>(A, S.ring, wv[j], v[j]);
+            }
+            if (e < n) {  // the rest, its loads still overlapped
+                uint32_t wv[kFlowApplyBatch];
+                FlowSlot<WIDE> v[kFlowApplyBatch];
+#pragma unroll
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) wv[j] = entry(min(e + j * nthr, n - 1u));
+#pragma unroll
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) v[j] = FlowSlot<WIDE>::load(A.rows, wv[j] >> S_EV);
 #pragma unroll
                 for (uint32_t j = 0; j < kFlowApplyBatch; j++)
-                    v[j] = e + j * nthr < n && wv[j] != kFlowDead ? __ldg(ev2 + (wv[j] >> (6u + LK)))
-                                                                   : make_uint2(kEvNone, kEvNone);
-#pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++) flow_put<K>(A, S.ring, wv[j], v[j]);
+                    if (e + j * nthr < n) flow_put<K, WIDE>(A, S.ring, wv[j], v[j]);
             }
             if (tma) fence_proxy_async_shared();  // ring writes before the tensor stores read them
             flow_bar(nthr);
             // every applier has read the step's arena entries (barrier): the
             // region is free for the walkers of later steps while the
             // appliers flush (release: those reads precede the hand-off)
-            U += S.scap[q];
+            U += S.scap[q] + S.slcap[q];
+            up += S.scap[q] + S.slcap[q];
+            if (up >= A.arena) up -= A.arena;
             if (at == 0) st_release_shared(&C.u_applied, U);
             // detectors [flush_lo, flush_hi) are final: write and clear them
             const uint32_t nd = st.w - st.z;
@@ -662,6 +819,9 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
             if (at == 0) {
                 C.done[slot] = 0u;
                 C.cnt[slot] = 0u;
+                C.left[slot] = 0u;
+#pragma unroll
+                for (uint32_t i = 0; i < kFlowBlocks / 4; i++) C.blk[slot][i] = 0u;
                 // release: every applier's ring writes of this step (ordered
                 // before by the barrier) and the counter resets precede the
                 // hand-off of the ring window and the step's slots
@@ -677,7 +837,7 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
 #define TMCS_FLOW_MAX_THREADS 1024
 #endif
 
-template <int K, int W, bool GA>
+template <int K, bool WIDE>
 __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __grid_constant__ FlowArgs A) {
     extern __shared__ __align__(128) uint64_t smem[];
     __shared__ FlowCtl C;
@@ -687,20 +847,27 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
     const uint32_t rows = A.window_mask + 1u;
     for (uint32_t i = tid; i < (rows + A.n_obs) * uint32_t(K); i += T_) S.ring[i] = 0ull;
     for (uint32_t i = tid; i < A.smem_tables * kTableWords; i += T_) S.stab[i] = __ldg(A.tables + i);
-    // region capacities: mean + 6 sigma + 64 of the step's events over K
+    // batches per step (prefix sum below) and region capacities: mean + 6 sigma + 64 of the step's events over K
     // chunks (Poisson-like counts), at most the arena; steps without items
     // hold none
     for (uint32_t i = tid; i < A.n_steps; i += T_) {
         const uint4 st = __ldg(A.steps + i);
-        const float mu = __ldg(A.step_events + i) * float(K);
+        const float2 ex = __ldg(A.step_events + i);
+        const float mu = ex.x * float(K), ml = ex.y * float(K);
         uint32_t cap = A.test_cap ? A.test_cap : uint32_t(ceilf(mu + 6.0f * sqrtf(mu) + 64.0f));
-        cap = st.y > st.x ? min(cap, A.arena) : 0u;
-        S.send[i] = st.y;
+        // put-aside streams: whole blocks, at most a quarter of the arena
+        uint32_t lcap = min((uint32_t(ceilf(ml + 6.0f * sqrtf(ml))) + 63u) & ~31u, (A.arena / 4u) & ~31u);
+        lcap = st.y > st.x ? min(lcap, 32u * kFlowBlocks) : 0u;
+        cap = st.y > st.x ? min(cap, A.arena - lcap) : 0u;
+        S.bend[i] = (st.y - st.x + 32u / uint32_t(K) - 1u) / (32u / uint32_t(K));
         S.scap[i] = cap;
+        S.slcap[i] = lcap;
     }
     if (tid < kFlowSlots) {
         C.done[tid] = 0u;
         C.cnt[tid] = 0u;
+        C.left[tid] = 0u;
+        for (uint32_t i = 0; i < kFlowBlocks / 4; i++) C.blk[tid][i] = 0u;
     }
     if (tid == 0) {
         C.next = 0u;
@@ -710,22 +877,30 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
         C.app_stop = 0u;
     }
     __syncthreads();
-    // region offsets: exclusive prefix sum of the capacities (warp 0)
-    if (tid < 32) {
-        const uint32_t per = (A.n_steps + 31u) / 32u, lo = tid * per, hi = min(A.n_steps, lo + per);
+    // region offsets: exclusive prefix sum of the capacities (warp 0);
+    // batches: inclusive prefix sum (warp 1)
+    if (tid < 64) {
+        const bool bat = tid >= 32;
+        const uint32_t l = tid & 31u;
+        const uint32_t per = (A.n_steps + 31u) / 32u, lo = min(A.n_steps, l * per), hi = min(A.n_steps, lo + per);
         uint32_t sum = 0;
-        for (uint32_t i = lo; i < hi; i++) sum += S.scap[i];
+        for (uint32_t i = lo; i < hi; i++) sum += bat ? S.bend[i] : S.scap[i] + S.slcap[i];
         uint32_t incl = sum;
         for (int o = 1; o < 32; o <<= 1) {
             const uint32_t v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-            if (int(tid) >= o) incl += v;
+            if (int(l) >= o) incl += v;
         }
         uint32_t run = incl - sum;
         for (uint32_t i = lo; i < hi; i++) {
-            S.soff[i] = run;
-            run += S.scap[i];
+            if (bat) {
+                run += S.bend[i];
+                S.bend[i] = run;
+            } else {
+                S.soff[i] = run;
+                run += S.scap[i] + S.slcap[i];
+            }
         }
-        if (tid == 31) S.soff[A.n_steps] = incl;
+        if (!bat && l == 31) S.soff[A.n_steps] = incl;
     }
     const uint64_t G = gridDim.x;
     const uint32_t nt = uint32_t((A.n_tiles - blockIdx.x + G - 1) / G);
@@ -733,9 +908,18 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
     const uint64_t rem = A.n_cols - last * K;
     const uint32_t nv_last = rem < uint64_t(K) ? uint32_t(rem) : uint32_t(K);
     __syncthreads();
-    if ((tid >> 5) >= A.walkers) flow_apply<K, GA>(A, S, C, nt, nv_last);
-    else if (A.smem_tables) flow_walk<K, W, true, GA>(A, S, C, nt, nv_last, S.stab);
-    else flow_walk<K, W, false, GA>(A, S, C, nt, nv_last, A.tables);
+    if ((tid >> 5) >= A.walkers) {
+        flow_apply<K, WIDE>(A, S, C, nt, nv_last);
+    } else {
+        const uint32_t lane = tid & 31u;
+        if (A.smem_tables) {
+            FlowWalker<K, true, WIDE> w{A, S, C, S.stab, lane, (1u << lane) - 1u};
+            w.run(nt, nv_last);
+        } else {
+            FlowWalker<K, false, WIDE> w{A, S, C, A.tables, lane, (1u << lane) - 1u};
+            w.run(nt, nv_last);
+        }
+    }
 }
 
 // ------------------------------------------------------------------- host
@@ -745,69 +929,48 @@ static int env_int_flow(const char *name, int dflt) {
     return (v && *v) ? std::atoi(v) : dflt;
 }
 
-// Philox calls per walker window: TMCS_FLOW_WINDOW (2 to 4) when set, else
-// the requested one (2 to 4), else 3
-static int flow_window(int window) {
-    const int wforce = env_int_flow("TMCS_FLOW_WINDOW", 0);
-    if (wforce >= 2 && wforce <= 4) return wforce;
-    return (window >= 2 && window <= 4) ? window : 3;
-}
-
 static size_t flow_fixed_bytes(const SigProgram &G, int sched, uint32_t n_obs, int K) {
     const SigSchedule &S = G.sched[sched];
     return flow_ring_bytes(S.window, n_obs, K) + flow_step_bytes(uint32_t(S.steps.size()));
 }
 
-bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out,
-                bool global_arena, int window) {
+bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out) {
     const SigProgram &G = c->sig;
     if (!G.ok || sched < 0 || size_t(sched) >= G.sched.size()) return false;
     const SigSchedule &S = G.sched[sched];
-    if (S.lag || S.steps.empty() || S.steps.size() > kFlowMaxSteps || S.step_events.size() != S.steps.size())
+    if (S.lag || S.rows.empty() || S.steps.empty() || S.steps.size() > kFlowMaxSteps ||
+        S.step_events.size() != 2 * S.steps.size())
         return false;
     if (K != 1 && K != 2 && K != 4 && K != 8 && K != 16) return false;
     if (threads < 64 || threads > TMCS_FLOW_MAX_THREADS || threads % 32 || appliers < 1 || appliers >= threads / 32)
         return false;
     // event words: slot << (6 + log2 K) | chunk << 6 | lane must fit 32 bits
-    // and never equal kFlowDead
-    if (uint64_t(G.n_event_slots) * 64u * uint64_t(K) >= (uint64_t(1) << 32)) return false;
+    if (G.n_compact_slots * 64u * uint64_t(K) >= (uint64_t(1) << 32)) return false;
+    // batches of a step are counted in 16 bits
+    for (const SigStep &t : S.steps)
+        if ((t.item_end - t.item_begin) / (32u / uint32_t(K)) >= 65000u) return false;
     const size_t fixed = flow_fixed_bytes(G, sched, uint32_t(c->n_obs), K);
     const size_t tabs = G.tables.size() * 4;
-    auto arena_for = [&](size_t used) {
-        uint32_t a = kFlowMaxArena;
-        while (a >= kFlowMinArena && used + size_t(a) * 4 > budget) a >>= 1;
-        return a;
+    // what is left of the budget, in entries
+    auto arena_for = [&](size_t used) -> uint32_t {
+        return used >= budget ? 0u : uint32_t(std::min<size_t>((budget - used) / 4, kFlowMaxArena)) & ~3u;
     };
     FlowShape s;
     s.sched = sched;
     s.K = K;
     s.threads = threads;
     s.appliers = appliers;
-    // global arena: tables stay in shared memory, the arena is an L2-resident
-    // slice per CTA of the library's scratch buffer
-    if (global_arena) {
-        if (fixed + tabs > budget) return false;
-        const int gforce = env_int_flow("TMCS_FLOW_GARENA", 0);  // tuning knob: global arena entries per CTA
-        s.arena = (gforce >= int(kFlowMinArena) && !(gforce & (gforce - 1))) ? uint32_t(gforce) : 65536u;
-        s.smem_tables = true;
-        s.smem = fixed + tabs;
-        s.garena_ctas = 0;  // set by the caller (resident CTAs)
-        s.window = flow_window(window);
-        s.global_arena = true;
-        *out = s;
-        return true;
-    }
-    s.window = flow_window(window);
+    // testing knob: Philox calls of every stream's first window (1 to 4)
+    const int wforce = env_int_flow("TMCS_FLOW_WINDOW", 0);
+    s.window = (wforce >= 1 && wforce <= 4) ? wforce : 0;
     // gap tables in shared memory when that still leaves an arena of 8192
     // entries, else read through L1
     s.smem_tables = arena_for(fixed + tabs) >= 8192u;
     s.arena = arena_for(fixed + (s.smem_tables ? tabs : 0));
     const int aforce = env_int_flow("TMCS_FLOW_ARENA", 0);  // tuning/testing knob: arena entries
-    if (aforce >= int(kFlowMinArena) && !(aforce & (aforce - 1)) && uint32_t(aforce) < s.arena)
-        s.arena = uint32_t(aforce);
+    if (aforce >= int(kFlowMinArena) && uint32_t(aforce) < s.arena) s.arena = uint32_t(aforce) & ~3u;
     if (s.arena < kFlowMinArena) return false;
     s.smem = fixed + (s.smem_tables ? tabs : 0) + size_t(s.arena) * 4;
-    if (s.smem > budget) return false;
     *out = s;
     return true;
 }
@@ -852,9 +1015,9 @@ static bool encode_det_map(CUtensorMap *map, uint64_t *det, uint64_t n_det, uint
            CUDA_SUCCESS;
 }
 
-template <int K, int W, bool GA>
+template <int K, bool WIDE>
 static cudaError_t flow_go(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t st) {
-    auto kern = flow_kernel<K, W, GA>;
+    auto kern = flow_kernel<K, WIDE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
@@ -863,38 +1026,25 @@ static cudaError_t flow_go(const FlowArgs &a, const FlowShape &s, int sms, cudaS
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, s.threads, s.smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
-    uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(a.n_tiles, uint64_t(sms) * uint64_t(per_sm)));
-    // a global arena holds one slice per CTA
-    if (GA) grid = std::min<uint64_t>(grid, s.garena_ctas);
-    // streams and steps are counted per CTA in 32 bits (flow_launch slices
-    // calls so that this holds)
-    const uint64_t tiles_per_cta = (a.n_tiles + grid - 1) / grid;
-    if (tiles_per_cta * uint64_t(a.n_steps) >= (uint64_t(1) << 31) ||
-        tiles_per_cta * (uint64_t(a.n_items) * uint64_t(K)) >= (uint64_t(1) << 31))
-        return cudaErrorInvalidValue;
+    const uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(a.n_tiles, uint64_t(sms) * uint64_t(per_sm)));
     kern<<<unsigned(grid), s.threads, s.smem, st>>>(a);
     return cudaGetLastError();
 }
 
-template <int W, bool GA>
-static cudaError_t flow_go_kg(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t st) {
-    switch (s.K) {
-    case 16: return flow_go<16, W, GA>(a, s, sms, st);
-    case 8: return flow_go<8, W, GA>(a, s, sms, st);
-    case 4: return flow_go<4, W, GA>(a, s, sms, st);
-    case 2: return flow_go<2, W, GA>(a, s, sms, st);
-    default: return flow_go<1, W, GA>(a, s, sms, st);
-    }
-}
-
-template <int W>
+template <bool WIDE>
 static cudaError_t flow_go_k(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t st) {
-    return a.garena ? flow_go_kg<W, true>(a, s, sms, st) : flow_go_kg<W, false>(a, s, sms, st);
+    switch (s.K) {
+    case 16: return flow_go<16, WIDE>(a, s, sms, st);
+    case 8: return flow_go<8, WIDE>(a, s, sms, st);
+    case 4: return flow_go<4, WIDE>(a, s, sms, st);
+    case 2: return flow_go<2, WIDE>(a, s, sms, st);
+    default: return flow_go<1, WIDE>(a, s, sms, st);
+    }
 }
 
 cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
                         const FlowCall &call, int sms, cudaStream_t st) {
-    if (!ds || s.sched < 0 || size_t(s.sched) >= G.sched.size() || !ds->step_events[s.sched])
+    if (!ds || s.sched < 0 || size_t(s.sched) >= G.sched.size() || !ds->rows[s.sched])
         return cudaErrorInvalidValue;
     const SigSchedule &S = G.sched[s.sched];
     FlowArgs a{};
@@ -902,18 +1052,27 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     a.tables = ds->tables;
     a.item_desc = reinterpret_cast<const uint4 *>(ds->item_desc[s.sched]);
     a.steps = reinterpret_cast<const uint4 *>(ds->steps[s.sched]);
-    a.step_events = ds->step_events[s.sched];
-    a.ev_ent = ds->ev_ent;
+    a.step_events = reinterpret_cast<const float2 *>(ds->step_events[s.sched]);
+    a.rows = ds->rows[s.sched];
     a.n_steps = uint32_t(S.steps.size());
-    a.n_items = uint32_t(S.items.size() / 2);
     a.window_mask = S.window - 1u;
     a.n_obs = n_obs;
     a.arena = s.arena;
     a.test_cap = uint32_t(std::max(0, env_int_flow("TMCS_TEST_FLOW_CAP", 0)));
+    a.calls = uint32_t(s.window);
+    a.pc1 = 0u;
+    for (const NoiseDesc &nd : G.noise) a.pc1 |= nd.kind == N_PC1 ? 1u : 0u;
+    a.near = 1u;
+    for (size_t t = kGapLen; t < G.tables.size(); t += kTableWords) {
+        float inv;
+        std::memcpy(&inv, &G.tables[t], 4);
+        if (!(std::fabs(inv) < kNearInv)) a.near = 0u;
+    }
     a.smem_tables = s.smem_tables ? uint32_t(G.tables.size() / kTableWords) : 0u;
     a.walkers = uint32_t(s.threads / 32 - s.appliers);
     a.key0 = call.key0;
     a.key1 = call.key1;
+    a.keys = philox_keys(call.key0, call.key1);
     a.ld = call.n_cols;
     // tensor-store flush: by default for tiles of 8 or more chunks (rows of
     // 64 bytes or more; narrower boxes measured slower than plain stores);
@@ -925,18 +1084,16 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     const int tma = env_int_flow("TMCS_FLOW_TMA", -1);
     if ((tma > 0 || (tma < 0 && s.K >= 8)) && encode_det_map(&a.tmap, call.det, G.n_det, call.n_cols, s.K, trows))
         a.tma_rows = trows;
-    if (s.garena_ctas) {
-        if (!call.scratch || call.scratch_bytes < size_t(s.garena_ctas) * s.arena * 4) return cudaErrorInvalidValue;
-        a.garena = call.scratch;
-    }
-    // A CTA counts its streams and its steps in 32 bits: a call with more
+    // A CTA counts its batches and its steps in 32 bits: a call with more
     // tiles per CTA than that allows runs as several launches over column
     // slices (each a multiple of the tile size, in column order).
-    const uint64_t per_tile_streams = uint64_t(a.n_items) * uint64_t(s.K);
+    const uint64_t ipb = 32u / uint64_t(s.K);
+    uint64_t per_tile_batches = 0;
+    for (const SigStep &t : S.steps) per_tile_batches += (t.item_end - t.item_begin + ipb - 1) / ipb;
     const uint64_t per_tile_steps = a.n_steps;
     const uint64_t lim = (uint64_t(1) << 31) - 1;
     const uint64_t max_tiles_per_cta =
-        std::max<uint64_t>(1, std::min(lim / std::max<uint64_t>(per_tile_streams, 1), lim / per_tile_steps) - 1);
+        std::max<uint64_t>(1, std::min(lim / std::max<uint64_t>(per_tile_batches, 1), lim / per_tile_steps) - 1);
     uint64_t slice_cols = max_tiles_per_cta * uint64_t(sms) * uint64_t(s.K);
     // testing knob: slices of this many tiles (so the sliced path runs at
     // sizes the tests can check)
@@ -953,12 +1110,7 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
         a.obs = call.obs ? call.obs + c0 : nullptr;
         a.vec_out = (reinterpret_cast<uintptr_t>(a.det) % 16 == 0 && a.ld % 2 == 0) ? 1u : 0u;
         a.status = call.status;
-        cudaError_t e;
-        switch (s.window) {
-        case 2: e = flow_go_k<2>(a, s, sms, st); break;
-        case 4: e = flow_go_k<4>(a, s, sms, st); break;
-        default: e = flow_go_k<3>(a, s, sms, st); break;
-        }
+        const cudaError_t e = G.wide ? flow_go_k<true>(a, s, sms, st) : flow_go_k<false>(a, s, sms, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

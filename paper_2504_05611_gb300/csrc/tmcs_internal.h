@@ -105,12 +105,10 @@ struct FlowShape {
     int K = 4;                // chunks per tile
     int threads = 1024;
     int appliers = 8;         // applier warps (the other warps walk)
-    int window = 3;           // Philox calls per walker window (2..4)
-    uint32_t arena = 0;       // event arena entries (power of two)
+    int window = 0;           // Philox calls of a stream's first window (1..4); 0: each item's own
+    uint32_t arena = 0;       // event arena entries
     bool smem_tables = false; // gap tables staged in shared memory
     size_t smem = 0;          // dynamic shared memory
-    bool global_arena = false;  // arena in a global scratch buffer (one slice of `arena` entries per CTA)
-    uint32_t garena_ctas = 0;   // CTAs the scratch buffer has slices for (global arena)
 };
 
 // One device copy of a program.
@@ -143,6 +141,7 @@ struct DeviceSig {
     const SigStep *steps[kSigMaxSchedules] = {};
     const float *step_events[kSigMaxSchedules] = {};
     const uint32_t *item_desc[kSigMaxSchedules] = {};
+    const uint32_t *rows[kSigMaxSchedules] = {};   // ring rows per compact event slot (SigSchedule::rows)
     const uint32_t *ev_ent = nullptr;
 };
 
@@ -153,15 +152,11 @@ struct DeviceSig {
 // schedules (lag 0) of at most kFlowMaxSteps steps.
 constexpr uint32_t kFlowMaxSteps = 1024;
 
-
-
 struct FlowCall {
     uint32_t key0 = 0, key1 = 0, first_chunk = 0;
     uint64_t n_cols = 0, last_mask = 0;
     uint64_t *det = nullptr, *obs = nullptr;
     uint32_t *status = nullptr;
-    uint32_t *scratch = nullptr;  // global arena slices (FlowShape::global_arena)
-    size_t scratch_bytes = 0;
 };
 
 // Per-device scratch of the library: a status word that kernels set when a
@@ -209,16 +204,44 @@ struct SigSchedule {
     // (units - 1) << 16 | descriptor << 22 (descriptor < 1024, table < 8192).
     std::vector<uint32_t> item_rec;
     std::vector<SigStep> steps;
-    // Expected events per 64-shot chunk of each step (sum over its items of
-    // 64 x units x p); the decoupled kernel sizes its event regions by it.
+    // Two numbers per step, expected per 64-shot chunk: the events that flip
+    // something (sum over its items of 64 x units x p x live share), and the
+    // streams that do not end in their first window; the decoupled kernel
+    // sizes the step's arena region by them.
     std::vector<float> step_events;
     // Walker descriptors of the decoupled kernel, 8 words per item (no
     // dependence on the seed): hi and lo of 0xCD9E8D57 x op index (Philox
-    // round 1), segment, first event slot, kind | npauli << 3 | paulis << 7
-    // | (units - 1) << 11 | step << 17, table | descriptor << 13, float bits
-    // of 1/log2(1-p) (the gap estimate), and the mask of Pauli indices that
-    // flip an output in some unit of the segment (bit k - 1 for index k).
+    // round 1), segment, first compact event slot, kind | npauli << 3 |
+    // classes per unit << 7 | (units - 1) << 11 | (first-window calls - 1)
+    // << 17 | table << 19, then the class of every Pauli index as nibbles
+    // (index k at bit 4 (k - 1) of the 64-bit word 5 | word 6 << 32; 0 = it
+    // flips nothing in any unit of the segment; in the two-row layout, where
+    // no segment has more than three classes, two bits per index in word 5;
+    // PAULI_CHANNEL_1 has three indices, and its descriptor index in word
+    // 6), and the float bits of 1/log2(1-p) (the gap estimate).
     std::vector<uint32_t> item_desc;
+    // Output lists of the compact event slots as rows of this schedule's
+    // ring (barrier schedules): row = detector mod window, or window +
+    // observable; unused entries name a spare row, window + observables,
+    // that nothing reads. A slot is one word of two 16-bit rows, or four
+    // words of eight (SigProgram::wide); bit 31 of the first word marks a
+    // longer list: kRowOverflow | word offset of a list [count, rows two per
+    // word] after the slots.
+    std::vector<uint32_t> rows;
+};
+
+constexpr uint32_t kRowOverflow = 0x80000000u;
+
+// Classes of one segment's Pauli indices (see SigProgram::compact).
+struct CompactItem {
+    uint32_t desc = 0, seg = 0;
+    uint64_t slot0 = 0;
+    uint64_t lut = 0;         // class of Pauli index k in nibble k - 1
+    uint32_t classes = 0;
+    uint8_t rep[16] = {};     // a Pauli index of class c at rep[c]
+    uint32_t calls = 1;       // Philox calls of a stream's first window
+    double events = 0;        // expected events per chunk that flip something
+    double left = 0;          // probability that a stream goes on after its first window
 };
 
 struct SigProgram {
@@ -242,6 +265,17 @@ struct SigProgram {
     std::vector<uint32_t> ev_base;   // per descriptor: index of its first event slot
     std::vector<uint32_t> ev_ent;
     uint32_t n_event_slots = 0;      // event slots (the overflow lists follow them in ev_ent)
+    // Compact event slots of the decoupled kernel: the Pauli indices of a
+    // segment that share their live generators (those with a non-empty
+    // output list in some unit of the segment) flip the same outputs in
+    // every unit, so a unit has one slot per class of indices instead of one
+    // per index (a surface-code DEPOLARIZE2 segment: 3 instead of 15). One
+    // CompactItem per segment that flips anything, in (descriptor, segment)
+    // order; slot = slot0 + unit * classes + (class - 1).
+    std::vector<struct CompactItem> compact;
+    std::vector<uint32_t> compact_of;  // first CompactItem index of each descriptor's segments (0xFFFFFFFF: none)
+    uint64_t n_compact_slots = 0;
+    bool wide = false;                 // eight rows per slot instead of two, up to 15 classes instead of 3
     double build_seconds = 0;
 };
 
@@ -315,11 +349,8 @@ int table_for_p(std::vector<uint32_t> &tables, std::vector<double> &table_p, dou
 void free_device_programs(tmcs_circuit *c);
 
 // Decoupled event-signature kernel (tmcs_flow.cu). flow_shape fills *out for
-// the given schedule, chunks per tile, CTA size, applier warps and walker
-// window (Philox calls per pass, 2 to 4; 0: 3; TMCS_FLOW_WINDOW overrides)
-// if that shape fits `budget` bytes of dynamic shared memory.
-bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out,
-                bool global_arena = false, int window = 0);
+// the given schedule, chunks per tile, CTA size and applier warps if that shape fits `budget` bytes of dynamic shared memory.
+bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out);
 #ifdef __CUDACC__
 cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
                         const FlowCall &call, int sms, cudaStream_t st);

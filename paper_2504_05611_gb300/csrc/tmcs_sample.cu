@@ -1630,7 +1630,7 @@ __global__ void gap_counts_kernel(const uint32_t *__restrict__ T, float inv, flo
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
         const uint32_t x = w[i];
         int g;
-        if (method == 0 && fabsf(inv) < kNearInv) g = gap_count_near<false>(T, inv, c32, x);
+        if (method == 0 && fabsf(inv) < kNearInv) g = gap_count_magic<false>(T, 0xFFFFFFFFu, inv, c32, x);
         else if (method <= 1) g = gap_count_est<false>(T, inv, c32, x);
         else g = gap_count(T, inv, x);
         out[i] = g;
@@ -1716,13 +1716,14 @@ static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
     const size_t b_tables = align256(G.tables.size() * 4);
     const size_t n_sched = G.sched.size();
     size_t b_items[kSigMaxSchedules] = {}, b_steps[kSigMaxSchedules] = {}, b_sev[kSigMaxSchedules] = {},
-           b_desc[kSigMaxSchedules] = {}, b_sched = 0;
+           b_desc[kSigMaxSchedules] = {}, b_rows[kSigMaxSchedules] = {}, b_sched = 0;
     for (size_t k = 0; k < n_sched; k++) {
         b_items[k] = align256(G.sched[k].item_rec.size() * 4);
         b_steps[k] = align256(G.sched[k].steps.size() * sizeof(SigStep));
         b_sev[k] = align256(G.sched[k].step_events.size() * sizeof(float));
         b_desc[k] = align256(G.sched[k].item_desc.size() * 4);
-        b_sched += b_items[k] + b_steps[k] + b_sev[k] + b_desc[k];
+        b_rows[k] = align256(G.sched[k].rows.size() * 4);
+        b_sched += b_items[k] + b_steps[k] + b_sev[k] + b_desc[k] + b_rows[k];
     }
     const size_t b_ent = align256(G.ev_ent.size() * 4);
     const size_t total = std::max<size_t>(b_noise + b_tables + b_sched + b_ent, 256);
@@ -1739,13 +1740,14 @@ static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
     const size_t o_noise = put(dn.data(), dn.size() * sizeof(NoiseDesc), b_noise);
     const size_t o_tables = put(G.tables.data(), G.tables.size() * 4, b_tables);
     size_t o_items[kSigMaxSchedules] = {}, o_steps[kSigMaxSchedules] = {}, o_sev[kSigMaxSchedules] = {},
-           o_desc[kSigMaxSchedules] = {};
+           o_desc[kSigMaxSchedules] = {}, o_rows[kSigMaxSchedules] = {};
     for (size_t k = 0; k < n_sched; k++) {
         const SigSchedule &S = G.sched[k];
         o_items[k] = put(S.item_rec.data(), S.item_rec.size() * 4, b_items[k]);
         o_steps[k] = put(S.steps.data(), S.steps.size() * sizeof(SigStep), b_steps[k]);
         o_sev[k] = put(S.step_events.data(), S.step_events.size() * sizeof(float), b_sev[k]);
         o_desc[k] = put(S.item_desc.data(), S.item_desc.size() * 4, b_desc[k]);
+        o_rows[k] = put(S.rows.data(), S.rows.size() * 4, b_rows[k]);
     }
     const size_t o_ent = put(G.ev_ent.data(), G.ev_ent.size() * 4, b_ent);
     void *base = nullptr;
@@ -1771,6 +1773,7 @@ static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
         ds.steps[k] = reinterpret_cast<const SigStep *>(b + o_steps[k]);
         ds.step_events[k] = reinterpret_cast<const float *>(b + o_sev[k]);
         ds.item_desc[k] = reinterpret_cast<const uint32_t *>(b + o_desc[k]);
+        if (!G.sched[k].rows.empty()) ds.rows[k] = reinterpret_cast<const uint32_t *>(b + o_rows[k]);
     }
     ds.ev_ent = reinterpret_cast<const uint32_t *>(b + o_ent);
     auto ins = c->dev_sig.emplace(dev, ds);
@@ -1924,18 +1927,15 @@ static LaunchShape make_shape_sig(const tmcs_circuit *c, uint64_t n_cols, const 
 // tile, `appliers` of its warps apply steps, the others walk. mode = 0 when
 // the shape does not fit.
 static LaunchShape make_shape_flow(const tmcs_circuit *c, uint64_t n_cols, const DeviceLimits &lim, int sched, int K,
-                                   int threads, int appliers, bool global_arena = false, int window = 0) {
+                                   int threads, int appliers) {
     LaunchShape s;
     s.mode = 0;
-    if (!flow_shape(c, sched, K, threads, appliers, lim.smem_optin - 1024, &s.flow, global_arena, window)) return s;
-    // a global arena has one slice per resident CTA (at most two per SM)
-    if (global_arena) s.flow.garena_ctas = uint32_t(2 * lim.sms);
+    if (!flow_shape(c, sched, K, threads, appliers, lim.smem_optin - 1024, &s.flow)) return s;
     s.mode = 7;
     s.sched = sched;
     s.K = K;
     s.threads = threads;
     s.warps = appliers;
-    s.group = global_arena ? 1 : 0;
     s.sms = lim.sms;
     s.smem = s.flow.smem;
     s.smem_tables = s.flow.smem_tables;
@@ -2034,34 +2034,6 @@ static cudaError_t launch_pipe(const SigArgs &a, const LaunchShape &s, cudaStrea
     return cudaGetLastError();
 }
 
-// ---- scratch of the decoupled kernel's global arena: one grow-only buffer
-// per (device, stream), so launches on different streams never share arena
-// slices (library-owned; allocated by the first call on that stream that
-// needs it, which must not be under stream capture)
-static std::mutex g_flow_scratch_mu;
-static std::map<std::pair<int, cudaStream_t>, std::pair<uint32_t *, size_t>> g_flow_scratch;
-
-static cudaError_t flow_scratch(cudaStream_t st, size_t bytes, uint32_t **out) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(g_flow_scratch_mu);
-    auto &slot = g_flow_scratch[{dev, st}];
-    if (slot.second < bytes) {
-        if (slot.first) {
-            // in-flight kernels may still use the old buffer
-            if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-            cudaFree(slot.first);
-            slot = {nullptr, 0};
-        }
-        void *p = nullptr;
-        if ((e = cudaMalloc(&p, bytes)) != cudaSuccess) return e;
-        slot = {static_cast<uint32_t *>(p), bytes};
-    }
-    *out = slot.first;
-    return cudaSuccess;
-}
-
 static cudaError_t launch(const KernelArgs &a0, const LaunchShape &s, cudaStream_t st,
                           const DeviceSig *ds = nullptr, const SigProgram *G = nullptr, uint32_t n_obs = 0) {
     if (s.mode == 7) {
@@ -2075,11 +2047,6 @@ static cudaError_t launch(const KernelArgs &a0, const LaunchShape &s, cudaStream
         call.det = a0.det;
         call.obs = a0.obs;
         call.status = a0.status;
-        if (s.flow.global_arena) {
-            call.scratch_bytes = size_t(s.flow.garena_ctas) * s.flow.arena * 4;
-            const cudaError_t e = flow_scratch(st, call.scratch_bytes, &call.scratch);
-            if (e != cudaSuccess) return e;
-        }
         return flow_launch(*G, n_obs, ds, s.flow, call, s.sms, st);
     }
     if (s.mode == 5 || s.mode == 6) {
@@ -2195,14 +2162,10 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
         for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
             if (c->sig.sched[sched].lag) continue;
             for (int K = 1; K <= 16; K *= 2)
-                for (int app : {8, 12, 16, 20, 24})
-                    for (int win : {3, 4}) {
-                        // shared-memory arena (the global-memory arena, a
-                        // tuning knob, measured no faster: its reads cost an
-                        // L2 trip)
-                        const LaunchShape cs = make_shape_flow(c, n_cols, lim, sched, K, 1024, app, false, win);
-                        if (cs.mode == 7 && (win == 3 || cs.flow.window == 4)) cands.push_back(cs);
-                    }
+                for (int app : {8, 12, 16, 20, 24}) {
+                    const LaunchShape cs = make_shape_flow(c, n_cols, lim, sched, K, 1024, app);
+                    if (cs.mode == 7) cands.push_back(cs);
+                }
         }
     // With a signature program the frame kernels are compared through their
     // heuristic shape only (they lost to kernel 4 on every measured
@@ -2290,8 +2253,7 @@ static LaunchShape choose_shape_sig(const tmcs_circuit *c, uint64_t n_cols, cons
         while (K > 1 && (K & (K - 1))) K--;
         const int tforce = env_int("TMCS_THREADS", 0);
         const int threads = (tforce >= 64 && tforce <= 1024 && tforce % 32 == 0) ? tforce : 1024;
-        return make_shape_flow(c, n_cols, lim, sched, K, threads, env_int("TMCS_FLOW_APPLIERS", 8),
-                               env_int("TMCS_FLOW_GLOBAL_ARENA", 0) > 0);
+        return make_shape_flow(c, n_cols, lim, sched, K, threads, env_int("TMCS_FLOW_APPLIERS", 8));
     }
     // tuning/testing knobs: TMCS_SIG_SCHED = schedule index among the barrier
     // schedules (0 = largest ring window), or among the pipelined ones with
@@ -2376,7 +2338,7 @@ static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t sh
             s = make_shape_sig(c, n_cols, lim, mdp.tuned_K, mdp.tuned_threads, mdp.tuned_sched);
         if (mdp.tuned_mode == 7 && ds) {
             const LaunchShape f = make_shape_flow(c, n_cols, lim, mdp.tuned_sched, mdp.tuned_K, mdp.tuned_threads,
-                                                  mdp.tuned_warps, mdp.tuned_group == 1, mdp.tuned_flow.window);
+                                                  mdp.tuned_warps);
             if (f.mode == 7) s = f;
         }
     }
@@ -3032,7 +2994,7 @@ int tmcs_launch_flow_shape(const tmcs_circuit *c, int *appliers, int *window, in
     const FlowShape f = flow ? it->second.tuned_flow : FlowShape();
     if (appliers) *appliers = flow ? f.appliers : 0;
     if (window) *window = flow ? f.window : 0;
-    if (global_arena) *global_arena = flow && f.global_arena ? 1 : 0;
+    if (global_arena) *global_arena = 0;
     if (arena_entries) *arena_entries = flow ? int(f.arena) : 0;
     return TMCS_OK;
 }

@@ -79,17 +79,218 @@ struct Pass {
 
 }  // namespace
 
-// Pauli indices of a segment that can flip an output: bit k - 1 is set when
-// event (unit, Pauli index k) has a non-empty output list for some unit of
-// the segment (slots slot0 .. slot0 + units * paulis - 1, unit-major). The
-// decoupled kernel drops the other events of the segment's streams before
-// they reach its arena: they flip nothing, so the result is unchanged.
-static uint32_t live_paulis(const SigProgram &G, uint32_t slot0, uint32_t units, uint32_t paulis) {
-    uint32_t m = 0;
-    for (uint32_t u = 0; u < units; u++)
-        for (uint32_t k = 0; k < paulis; k++)
-            if (G.ev_ent[2 * (size_t(slot0) + size_t(u) * paulis + k)] != kEvNone) m |= 1u << k;
-    return m;
+// Output list of event slot k (entries as in SigProgram::ev_ent).
+static void event_list(const SigProgram &G, size_t k, std::vector<uint32_t> &v) {
+    const uint32_t w0 = G.ev_ent[2 * k], w1 = G.ev_ent[2 * k + 1];
+    v.clear();
+    if (w0 == kEvNone) return;
+    if (w0 & kEvOverflow) {
+        const size_t off = w0 & ~kEvOverflow;
+        v.assign(G.ev_ent.begin() + off, G.ev_ent.begin() + off + w1);
+        return;
+    }
+    v.push_back(w0);
+    if (w1 != kEvNone) v.push_back(w1);
+}
+
+// Words of a compact event slot.
+static size_t slot_words(const SigProgram &G) { return G.wide ? 4 : 1; }
+
+// Philox calls (two draws each) of the first window of a stream that expects
+// `lambda` events (Poisson), and the probability that it goes on after it.
+// A walker runs the window for 32 streams at once and finishes the streams
+// that go on (2w or more events) 32 at a time, for as many calls as the
+// longest of the 32 needs. The costs below (warp-instructions: a call of the
+// window; setting streams aside, when any of the 32 goes on; a finishing
+// pass and each of its calls) are fitted to the d=29 and d=11 surface-code
+// workloads at windows of 1 to 4 calls; at 4.1 expected events (p = 1e-3)
+// windows of 2 / 3 / 4 calls measured 491 / 296 / 310 ns per chunk, at 0.41
+// (p = 1e-4) windows of 1 / 2 calls 175 / 181.
+static uint32_t first_window_calls(double lambda, double *left) {
+    const int kMax = 64;
+    double pmf[kMax], tail[kMax + 1];  // tail[k] = P(X >= k)
+    double term = std::exp(-lambda);
+    tail[0] = 1.0;
+    for (int k = 0; k < kMax; k++) {
+        pmf[k] = term;
+        tail[k + 1] = std::max(0.0, tail[k] - term);
+        term *= lambda / double(k + 1);
+    }
+    double best = 1e300;
+    uint32_t w_best = 1;
+    for (uint32_t w = 1; w <= 4; w++) {
+        const double p = tail[2 * w];
+        double calls = 1.0;
+        for (int k = int(2 * w) + 2; k <= kMax && 32.0 * tail[k] > 0.5 * p; k += 2) calls += 1.0;
+        const double cost = 170.0 * w + 60.0 * (1.0 - std::pow(1.0 - p, 32.0)) + p * (300.0 + 230.0 * calls);
+        if (cost < best) {
+            best = cost;
+            w_best = w;
+            *left = p;
+        }
+    }
+    return w_best;
+}
+
+// Share of a noise kind's drawn Pauli indices whose class is not 0.
+static double live_share(const NoiseDesc &nd, uint64_t lut) {
+    if (nd.kind == N_PC1) {
+        const double q = 1.0 / 4294967296.0, t1 = nd.t1 * q, t2 = nd.t2 * q;
+        return ((lut & 15u) ? t1 : 0.0) + ((lut >> 8 & 15u) ? std::max(0.0, t2 - t1) : 0.0) +
+               ((lut >> 4 & 15u) ? 1.0 - t2 : 0.0);
+    }
+    const uint32_t n = sig_paulis(nd.kind);
+    uint32_t live = 0;
+    for (uint32_t k = 0; k < n; k++) live += (lut >> (4 * k) & 15u) ? 1u : 0u;
+    return double(live) / double(n);
+}
+
+// Words 5 and 6 of an item's walker descriptor (see SigSchedule::item_desc).
+static void lut_words(const SigProgram &G, const CompactItem &ci, uint32_t *lo, uint32_t *hi) {
+    if (G.wide) {
+        *lo = uint32_t(ci.lut);
+        *hi = uint32_t(ci.lut >> 32);
+    } else {
+        *lo = *hi = 0;
+        for (uint32_t k = 0; k < 15; k++) *lo |= uint32_t(ci.lut >> (4 * k) & 3u) << (2 * k);
+    }
+    if (G.noise[ci.desc].kind == N_PC1) *hi = ci.desc;
+}
+
+// Classes and compact event slots of every segment that flips anything.
+static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
+    G.compact.clear();
+    G.compact_of.assign(G.noise.size(), 0xFFFFFFFFu);
+    uint64_t slots = 0, long_lists = 0;
+    uint32_t max_classes = 0;
+    for (uint32_t di = 0; di < G.noise.size(); di++) {
+        const NoiseDesc &nd = G.noise[di];
+        const uint32_t ng = sig_gens(nd.kind), KP = sig_paulis(nd.kind);
+        G.compact_of[di] = uint32_t(G.compact.size());
+        for (uint32_t s = 0; s < nd.n_seg; s++) {
+            const uint32_t u0 = s * kSegUnits, u1 = std::min(nd.n_units, u0 + kSegUnits);
+            uint32_t live = 0;
+            for (uint32_t u = u0; u < u1; u++)
+                for (uint32_t g = 0; g < ng; g++)
+                    if (G.gen_off[nd.tgt_off + u * ng + g] != G.gen_off[nd.tgt_off + u * ng + g + 1]) live |= 1u << g;
+            CompactItem it;
+            it.desc = di;
+            it.seg = s;
+            it.slot0 = slots;
+            uint8_t cls[16] = {};  // class by live generator set
+            for (uint32_t k = 1; k <= KP; k++) {
+                const uint32_t m = sig_mask(nd.kind, k) & live;
+                if (!m) continue;
+                if (!cls[m]) {
+                    cls[m] = uint8_t(++it.classes);
+                    it.rep[it.classes] = uint8_t(k);
+                }
+                it.lut |= uint64_t(cls[m]) << (4 * (k - 1));
+            }
+            const double lambda = 64.0 * double(u1 - u0) * table_p[nd.table];
+            it.calls = first_window_calls(lambda, &it.left);
+            it.events = lambda * live_share(nd, it.lut);
+            max_classes = std::max(max_classes, it.classes);
+            slots += uint64_t(u1 - u0) * it.classes;
+            for (uint32_t u = u0; u < u1; u++)
+                for (uint32_t c = 1; c <= it.classes; c++) {
+                    const size_t k = G.ev_base[di] + size_t(u) * KP + (it.rep[c] - 1u);
+                    if (G.ev_ent[2 * k] != kEvNone && (G.ev_ent[2 * k] & kEvOverflow)) long_lists++;
+                }
+            G.compact.push_back(it);
+        }
+    }
+    G.n_compact_slots = slots;
+    // a list of three or more outputs costs the appliers a dependent read
+    // of its own in the two-row layout: eight rows per slot when more than
+    // one slot in sixteen has one (BB codes: about half; surface codes: a
+    // few per cent), or when a segment has more classes than its layout holds
+    G.wide = long_lists * 16 > slots || max_classes > 3;
+}
+
+static uint32_t row_of(uint32_t entry, uint32_t W) {
+    const uint32_t idx = entry & 0x1FFFFFFFu;
+    return (entry & (1u << 29)) ? W + idx : (idx & (W - 1u));
+}
+
+// Row table of a barrier schedule (see SigSchedule::rows).
+static bool build_rows(const SigProgram &G, uint64_t O, SigSchedule &S) {
+    const size_t wpr = slot_words(G);
+    if (uint64_t(S.window) + O >= 0x7FFFu || G.n_compact_slots * wpr >= (uint64_t(1) << 30)) return false;
+    const uint32_t spare = S.window + uint32_t(O), none = spare | (spare << 16);
+    S.rows.assign(G.n_compact_slots * wpr, none);
+    std::vector<uint32_t> v;
+    for (const CompactItem &it : G.compact) {
+        const NoiseDesc &nd = G.noise[it.desc];
+        const uint32_t KP = sig_paulis(nd.kind);
+        const uint32_t u0 = it.seg * kSegUnits, units = std::min(kSegUnits, nd.n_units - u0);
+        for (uint32_t u = 0; u < units; u++)
+            for (uint32_t c = 1; c <= it.classes; c++) {
+                event_list(G, G.ev_base[it.desc] + size_t(u0 + u) * KP + (it.rep[c] - 1u), v);
+                const size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr;
+                for (uint32_t &e : v) e = row_of(e, S.window);
+                size_t to = at;
+                if (v.size() > 2 * wpr) {
+                    to = S.rows.size() + 1;
+                    if (to + v.size() / 2 + 1 >= (uint64_t(1) << 31)) return false;
+                    S.rows[at] = kRowOverflow | uint32_t(S.rows.size());
+                    S.rows.push_back(uint32_t(v.size()));
+                    S.rows.resize(S.rows.size() + (v.size() + 1) / 2, none);
+                }
+                for (size_t x = 0; x < v.size(); x++) {
+                    uint32_t &w = S.rows[to + x / 2];
+                    w = (x & 1) ? (w & 0xFFFFu) | (v[x] << 16) : (w & 0xFFFF0000u) | v[x];
+                }
+            }
+    }
+    while (S.rows.size() % 4) S.rows.push_back(none);
+    return true;
+}
+
+// Checks a barrier schedule's row table: every Pauli index of every unit
+// finds, through its segment's classes, exactly its own output list as rows
+// of the ring (an index of class 0 flips nothing).
+static std::string validate_rows(const SigProgram &G, uint64_t O, const SigSchedule &S) {
+    const size_t wpr = slot_words(G);
+    if (S.rows.size() < G.n_compact_slots * wpr || uint64_t(S.window) + O >= 0x7FFFu) return "row table size";
+    const uint32_t spare = S.window + uint32_t(O);
+    std::vector<uint32_t> v, r, prev;
+    for (const CompactItem &it : G.compact) {
+        const NoiseDesc &nd = G.noise[it.desc];
+        const uint32_t KP = sig_paulis(nd.kind);
+        const uint32_t u0 = it.seg * kSegUnits, units = std::min(kSegUnits, nd.n_units - u0);
+        if (it.slot0 + uint64_t(units) * it.classes > G.n_compact_slots) return "compact slot";
+        for (uint32_t u = 0; u < units; u++)
+            for (uint32_t k = 1; k <= KP; k++) {
+                const size_t ek = G.ev_base[it.desc] + size_t(u0 + u) * KP + (k - 1u);
+                const uint32_t c = uint32_t(it.lut >> (4 * (k - 1))) & 15u;
+                if (c > it.classes) return "event class";
+                if (!c) {
+                    if (G.ev_ent[2 * ek] != kEvNone) return "event class";
+                    continue;
+                }
+                event_list(G, ek, v);
+                const uint32_t *w = &S.rows[(it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr];
+                size_t n = 2 * wpr;
+                if (w[0] & kRowOverflow) {
+                    const size_t off = w[0] & ~kRowOverflow;
+                    if (off < G.n_compact_slots * wpr || off >= S.rows.size()) return "row list";
+                    n = S.rows[off];
+                    w = S.rows.data() + off + 1;
+                    if (n <= 2 * wpr || off + 1 + (n + 1) / 2 > S.rows.size()) return "row list";
+                }
+                size_t x = 0;
+                for (; x < n; x++) {
+                    const uint32_t row = (w[x / 2] >> (16 * (x & 1))) & 0xFFFFu;
+                    if (row == spare) break;
+                    if (x >= v.size() || row != row_of(v[x], S.window)) return "event row";
+                }
+                if (x != v.size()) return "event row";
+                for (; x < n + (n & 1); x++)  // the rest names the spare row
+                    if (((w[x / 2] >> (16 * (x & 1))) & 0xFFFFu) != spare) return "event row";
+            }
+    }
+    return std::string();
 }
 
 // Checks every invariant the signature kernels rely on, after each build:
@@ -160,7 +361,7 @@ static std::string validate_signature_program(const SigProgram &G, uint64_t D, u
         const uint32_t W = S.window;
         if (W < 256 || (W & (W - 1)) || S.lag > uint32_t(kSigMaxLag) || (S.lag && W > 16384)) return "schedule shape";
         if (S.item_rec.size() != 4 * n_items || S.steps.empty()) return "schedule size";
-        if (S.step_events.size() != S.steps.size()) return "step event counts";
+        if (S.step_events.size() != 2 * S.steps.size()) return "step event counts";
         if (S.item_desc.size() != 8 * n_items || S.steps.size() > (1u << 15)) return "walker descriptors size";
         std::vector<uint64_t> lo(n_items), hi(n_items);
         for (size_t k = 0; k < n_items; k++) {
@@ -175,14 +376,16 @@ static std::string validate_signature_program(const SigProgram &G, uint64_t D, u
             // walker descriptor: the indices the decoupled kernel forms from it
             const uint32_t *wd = &S.item_desc[8 * k];
             const uint64_t m = uint64_t(0xCD9E8D57u) * nd.op_index;
-            const uint32_t step = wd[4] >> 17;
-            if (wd[0] != uint32_t(m >> 32) || wd[1] != uint32_t(m) || wd[2] != sg || wd[3] != r[2] ||
+            const CompactItem *ci = nullptr;
+            if (G.compact_of[di] + sg < G.compact.size()) ci = &G.compact[G.compact_of[di] + sg];
+            if (!ci || ci->desc != di || ci->seg != sg) return "compact item";
+            uint32_t lut_lo, lut_hi;
+            lut_words(G, *ci, &lut_lo, &lut_hi);
+            if (wd[0] != uint32_t(m >> 32) || wd[1] != uint32_t(m) || wd[2] != sg || wd[3] != uint32_t(ci->slot0) ||
                 (wd[4] & 7u) != nd.kind || ((wd[4] >> 3) & 15u) != (nd.kind == 3u ? 15u : nd.kind == 2u ? 3u : 1u) ||
-                ((wd[4] >> 7) & 15u) != sig_paulis(nd.kind) || ((wd[4] >> 11) & 63u) != units - 1 ||
-                step >= S.steps.size() || k < S.steps[step].item_begin || k >= S.steps[step].item_end ||
-                (wd[5] & 0x1FFFu) != nd.table || (wd[5] >> 13) != di ||
-                wd[6] != G.tables[size_t(nd.table) * kTableWords + kGapLen] ||
-                wd[7] != live_paulis(G, r[2], units, sig_paulis(nd.kind)))
+                ((wd[4] >> 7) & 15u) != ci->classes || ((wd[4] >> 11) & 63u) != units - 1 ||
+                (wd[4] >> 19) != nd.table || wd[5] != lut_lo || wd[6] != lut_hi ||
+                wd[7] != G.tables[size_t(nd.table) * kTableWords + kGapLen])
                 return "walker descriptor";
             lo[k] = seg_lo[seg0[di] + sg];
             hi[k] = seg_hi[seg0[di] + sg];
@@ -210,6 +413,10 @@ static std::string validate_signature_program(const SigProgram &G, uint64_t D, u
                 for (size_t u = v0; u <= v; u++) h = std::max<uint64_t>(h, shi[u % ns] + (u / ns) * D);
                 if (h - (S.steps[v0 % ns].flush_lo + (v0 / ns) * D) > W) return "ring too small for its lag";
             }
+        if (!S.rows.empty()) {
+            const std::string bad = validate_rows(G, O, S);
+            if (!bad.empty()) return bad;
+        }
     }
     return std::string();
 }
@@ -551,6 +758,7 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
     // capped by D), and up to two more schedules halve it while feasible
     // (a smaller ring lets more chunks or CTAs share an SM; the autotuner
     // picks).
+    build_compact(G, table_p);
     uint64_t need = 0;
     for (size_t i = 0; i < n_items; i++)
         if (dmin[i] != 0xFFFFFFFFu) need = std::max<uint64_t>(need, uint64_t(dmax[i]) - sufmin[i] + 1);
@@ -596,12 +804,16 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
             S.items[2 * k] = items[2 * perm[k]];
             S.items[2 * k + 1] = items[2 * perm[k] + 1];
         }
-        // expected events per chunk of each step: 64 trials per unit at the
-        // op's probability (the decoupled kernel sizes its event regions)
+        // expected live events and unfinished streams per chunk of each step
         for (const SigStep &st : S.steps) {
-            double ev = 0;
-            for (uint32_t k = st.item_begin; k < st.item_end; k++) ev += 64.0 * cost(perm[k]);
+            double ev = 0, left = 0;
+            for (uint32_t k = st.item_begin; k < st.item_end; k++) {
+                const CompactItem &ci = G.compact[G.compact_of[S.items[2 * k]] + S.items[2 * k + 1]];
+                ev += ci.events;
+                left += ci.left;
+            }
             S.step_events.push_back(float(ev));
+            S.step_events.push_back(float(left));
         }
         // walker descriptors of the decoupled kernel (see SigSchedule)
         for (uint32_t t = 0; t < S.steps.size(); t++)
@@ -609,15 +821,16 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
                 const uint32_t di = S.items[2 * k], sg = S.items[2 * k + 1];
                 const NoiseDesc &nd = G.noise[di];
                 const uint32_t units = std::min(kSegUnits, nd.n_units - sg * kSegUnits);
+                const CompactItem &ci = G.compact[G.compact_of[di] + sg];
                 const uint64_t m = uint64_t(0xCD9E8D57u) * nd.op_index;
                 const uint32_t npauli = nd.kind == 3u ? 15u : nd.kind == 2u ? 3u : 1u;
-                uint32_t inv_bits = G.tables[size_t(nd.table) * kTableWords + kGapLen];
-                const uint32_t slot0 = G.ev_base[di] + sg * kSegUnits * sig_paulis(nd.kind);
-                const uint32_t w[8] = {uint32_t(m >> 32), uint32_t(m), sg, slot0,
-                                       nd.kind | (npauli << 3) | (sig_paulis(nd.kind) << 7) | ((units - 1) << 11) |
-                                           (t << 17),
-                                       nd.table | (di << 13), inv_bits,
-                                       live_paulis(G, slot0, units, sig_paulis(nd.kind))};
+                uint32_t lut_lo, lut_hi;
+                lut_words(G, ci, &lut_lo, &lut_hi);
+                const uint32_t w[8] = {uint32_t(m >> 32), uint32_t(m), sg, uint32_t(ci.slot0),
+                                       nd.kind | (npauli << 3) | (ci.classes << 7) | ((units - 1) << 11) |
+                                           ((ci.calls - 1) << 17) | (nd.table << 19),
+                                       lut_lo, lut_hi,
+                                       G.tables[size_t(nd.table) * kTableWords + kGapLen]};
                 S.item_desc.insert(S.item_desc.end(), w, w + 8);
             }
         // device item records (the walk reads one 16-byte record per stream)
@@ -639,6 +852,8 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
             G.sched.clear();
             return TMCS_OK;
         }
+        // no row table: the decoupled kernel does not run this schedule
+        if (!build_rows(G, O, G.sched.back())) G.sched.back().rows.clear();
         if (W == 1024) break;
     }
 
@@ -695,9 +910,10 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
         } else if (what == "window" && !G.sched.empty()) {
             G.sched[0].window = 256;  // steps cut for a larger ring
         } else if (what == "live" && !G.sched.empty()) {
-            // drop a Pauli index that flips something from one item's mask
+            // a wrong class for a Pauli index that flips something (class 1
+            // becomes 0: the walkers would drop its events)
             std::vector<uint32_t> &wd = G.sched[0].item_desc;
-            for (size_t k = 7; k < wd.size(); k += 8)
+            for (size_t k = 5; k < wd.size(); k += 8)
                 if (wd[k]) {
                     wd[k] &= wd[k] - 1u;
                     break;
