@@ -336,7 +336,7 @@ namespace tmcs {
 // Host side (tmcs_host.cpp)
 void set_error(const std::string &msg);
 int fail(int code, const std::string &msg);
-int compile(tmcs_circuit *c, uint32_t flags, bool meas);
+int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped = true);
 int reference_record(const tmcs_circuit *c, std::vector<uint8_t> *rec);
 int build_measurement_program(tmcs_circuit *c);
 int gap_table(double p, uint32_t *t);
