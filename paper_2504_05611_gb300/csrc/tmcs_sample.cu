@@ -2173,9 +2173,25 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
                     cudaStream_t st, LaunchShape *best, const DeviceSig *ds) {
     const Program &P = c->prog;
     std::vector<LaunchShape> cands;
-    // every schedule of the signature program (barrier kernel for lag 0,
-    // pipelined kernel otherwise) x chunks per CTA x CTA size
+    // decoupled kernel: every barrier schedule x chunks per tile x applier
+    // warps, 1024 threads. Circuits whose events flip many outputs (BB codes:
+    // weight-6 checks, several observables) want more applier warps than the
+    // surface-code ones.
     if (ds)
+        for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
+            if (c->sig.sched[sched].lag) continue;
+            for (int K = 2; K <= 16; K *= 2)
+                for (int app : {8, 12, 16, 20, 24}) {
+                    const LaunchShape cs = make_shape_flow(c, n_cols, lim, sched, K, 1024, app);
+                    if (cs.mode == 7) cands.push_back(cs);
+                }
+        }
+    // circuits it does not fit: every schedule of the signature program
+    // (barrier kernel for lag 0, pipelined kernel otherwise) x chunks per CTA
+    // x CTA size. Where both fit these lost on every measured workload (d=29
+    // 21.1 against 9.4 ms, BB144 teleport 6.9 against 2.6), so they are not
+    // timed there.
+    if (ds && cands.empty())
         for (int sched = 0; sched < int(c->sig.sched.size()); sched++)
             for (int K = 1; K <= 16; K *= 2) {
                 if (!sig_fits(c, lim, K, sched)) break;
@@ -2184,25 +2200,10 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
                     if (sig_shape_fits(cs, lim)) cands.push_back(cs);
                 }
             }
-    // decoupled kernel: every barrier schedule x chunks per tile x applier
-    // warps x walker window (3 or 4 Philox calls), 1024 threads. Circuits
-    // whose events flip many outputs (BB codes: weight-6 checks, several
-    // observables) want more applier warps than the surface-code ones.
-    if (ds)
-        for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
-            if (c->sig.sched[sched].lag) continue;
-            for (int K = 1; K <= 16; K *= 2)
-                for (int app : {8, 12, 16, 20, 24}) {
-                    const LaunchShape cs = make_shape_flow(c, n_cols, lim, sched, K, 1024, app);
-                    if (cs.mode == 7) cands.push_back(cs);
-                }
-        }
-    // With a signature program the frame kernels are compared through their
-    // heuristic shape only (they lost to kernel 4 on every measured
-    // workload); without one, every feasible frame shape is timed.
-    if (ds) {
-        cands.push_back(choose_shape_cta(P, n_cols, lim));
-    } else {
+    // The frame kernels: with a signature program only when it fits nowhere
+    // (they lost to the signature kernels on every measured workload), then
+    // every feasible frame shape.
+    if (cands.empty()) {
         for (int K = 1; K <= 16; K *= 2) {
             if (!shape_fits(P, lim, K)) break;
             for (int threads : {128, 256, 512}) cands.push_back(make_shape(P, n_cols, K, threads));
@@ -2313,6 +2314,37 @@ static LaunchShape choose_shape_sig(const tmcs_circuit *c, uint64_t n_cols, cons
     return s;
 }
 
+// Shape of a call that nothing has been timed for (too few columns for the
+// autotuner, or under stream capture): the decoupled kernel. A CTA runs its
+// tiles one after another, so the time goes as tiles per CTA times a tile's
+// time, which measured as about one chunk's worth of fixed latency (the
+// steps' hand-overs) plus K chunks; K minimises that product. Measured
+// (best K / best time / time at the K chosen, us): d=29, 677 chunks 2 / 384
+// / 384; d=29, 150 chunks 1 / 126 / 126; d=11, 1563 chunks 4 / 74 / 74;
+// d=11, 157 chunks 2 / 44 / 45; BB144 teleport, 1563 chunks 4 / 141 / 156.
+// The largest ring that fits: fewer steps, so fewer hand-overs (d=29, 677
+// chunks, K = 4: ring 4096 402, 2048 485). Events of the eight-row layout
+// cost the appliers more, so they get more warps. mode = 0: no shape fits.
+static LaunchShape choose_shape_flow(const tmcs_circuit *c, uint64_t n_cols, const DeviceLimits &lim) {
+    LaunchShape best;
+    best.mode = 0;
+    uint64_t best_cost = 0;
+    for (int K = 1; K <= 16; K *= 2) {
+        const uint64_t tiles = (n_cols + uint64_t(K) - 1) / uint64_t(K);
+        const uint64_t cost = (tiles + uint64_t(lim.sms) - 1) / uint64_t(lim.sms) * uint64_t(K + 1);
+        if (best.mode && cost >= best_cost) continue;
+        for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
+            if (c->sig.sched[sched].lag) continue;
+            const LaunchShape s = make_shape_flow(c, n_cols, lim, sched, K, 1024, c->sig.wide ? 16 : 12);
+            if (s.mode != 7) continue;
+            best = s;
+            best_cost = cost;
+            break;
+        }
+    }
+    return best;
+}
+
 static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t shots, uint64_t seed,
                         uint64_t *det, uint64_t *obs, void *stream, bool fault_mode = false,
                         uint64_t fault_first = 0) {
@@ -2362,6 +2394,10 @@ static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t sh
     if (!forced && !fault_mode) {
         std::lock_guard<std::mutex> lock(c->mu);
         DeviceProgram &mdp = c->dev[dp->device];
+        if (mdp.tuned_mode == 0 && ds) {
+            const LaunchShape f = choose_shape_flow(c, n_cols, lim);
+            if (f.mode == 7) s = f;
+        }
         if (mdp.tuned_mode == 3) s = make_shape(P, n_cols, mdp.tuned_K, mdp.tuned_threads);
         if (mdp.tuned_mode == 4) s = make_shape_w(P, n_cols, mdp.tuned_K, mdp.tuned_warps, mdp.tuned_group);
         if ((mdp.tuned_mode == 5 || mdp.tuned_mode == 6) && ds)
