@@ -381,10 +381,9 @@ int tmcs_launch_shape(const tmcs_circuit *c, int *mode, int *chunks, int *thread
 
 /*
  * The decoupled kernel's part of the chosen shape (mode 7; zeros otherwise):
- * applier warps, Philox calls of a stream's first window when one is forced
- * (0: every item's own, chosen from its noise), global_arena (always 0: the
- * event arena is in shared memory), and the arena's entries (per CTA). Together with
- * tmcs_launch_shape this fixes the launch (for reports and for forcing the
+ * applier warps, Philox calls of a stream's first window, global_arena (always
+ * 0: the event arena is in shared memory), and the arena's entries (per CTA).
+ * Together with tmcs_launch_shape this fixes the launch (for reports and for forcing the
  * same shape with the tuning knobs). Any pointer may be NULL.
  * Errors: as tmcs_launch_shape.
  */

@@ -105,7 +105,7 @@ struct FlowShape {
     int K = 4;                // chunks per tile
     int threads = 1024;
     int appliers = 8;         // applier warps (the other warps walk)
-    int window = 0;           // Philox calls of a stream's first window (1..4); 0: each item's own
+    int window = 1;           // Philox calls of a stream's first window (1..4)
     uint32_t arena = 0;       // event arena entries
     bool smem_tables = false; // gap tables staged in shared memory
     size_t smem = 0;          // dynamic shared memory
@@ -212,8 +212,7 @@ struct SigSchedule {
     // Walker descriptors of the decoupled kernel, 8 words per item (no
     // dependence on the seed): hi and lo of 0xCD9E8D57 x op index (Philox
     // round 1), segment, first compact event slot, kind | npauli << 3 |
-    // classes per unit << 7 | (units - 1) << 11 | (first-window calls - 1)
-    // << 17 | table << 19, then the class of every Pauli index as nibbles
+    // classes per unit << 7 | (units - 1) << 11 | table << 19, then the class of every Pauli index as nibbles
     // (index k at bit 4 (k - 1) of the 64-bit word 5 | word 6 << 32; 0 = it
     // flips nothing in any unit of the segment; in the two-row layout, where
     // no segment has more than three classes, two bits per index in word 5;
@@ -239,9 +238,8 @@ struct CompactItem {
     uint64_t lut = 0;         // class of Pauli index k in nibble k - 1
     uint32_t classes = 0;
     uint8_t rep[16] = {};     // a Pauli index of class c at rep[c]
-    uint32_t calls = 1;       // Philox calls of a stream's first window
     double events = 0;        // expected events per chunk that flip something
-    double left = 0;          // probability that a stream goes on after its first window
+    double left[5] = {};      // probability that a stream goes on after a first window of 1..4 calls
 };
 
 struct SigProgram {
@@ -275,6 +273,7 @@ struct SigProgram {
     std::vector<struct CompactItem> compact;
     std::vector<uint32_t> compact_of;  // first CompactItem index of each descriptor's segments (0xFFFFFFFF: none)
     uint64_t n_compact_slots = 0;
+    uint32_t window_calls = 1;         // Philox calls of a stream's first window in the decoupled kernel
     bool wide = false;                 // eight rows per slot instead of two, up to 15 classes instead of 3
     double build_seconds = 0;
 };

@@ -96,40 +96,31 @@ static void event_list(const SigProgram &G, size_t k, std::vector<uint32_t> &v) 
 // Words of a compact event slot.
 static size_t slot_words(const SigProgram &G) { return G.wide ? 4 : 1; }
 
-// Philox calls (two draws each) of the first window of a stream that expects
-// `lambda` events (Poisson), and the probability that it goes on after it.
-// A walker runs the window for 32 streams at once and finishes the streams
-// that go on (2w or more events) 32 at a time, for as many calls as the
-// longest of the 32 needs. The costs below (warp-instructions: a call of the
-// window; setting streams aside, when any of the 32 goes on; a finishing
-// pass and each of its calls) are fitted to the d=29 and d=11 surface-code
-// workloads at windows of 1 to 4 calls; at 4.1 expected events (p = 1e-3)
-// windows of 2 / 3 / 4 calls measured 491 / 296 / 310 ns per chunk, at 0.41
-// (p = 1e-4) windows of 1 / 2 calls 175 / 181.
-static uint32_t first_window_calls(double lambda, double *left) {
-    const int kMax = 64;
-    double pmf[kMax], tail[kMax + 1];  // tail[k] = P(X >= k)
+// Distribution of a stream's events (Poisson with mean lambda): P(X >= k).
+static void poisson_tail(double lambda, std::vector<double> &tail) {
+    tail.assign(66, 0.0);
     double term = std::exp(-lambda);
     tail[0] = 1.0;
-    for (int k = 0; k < kMax; k++) {
-        pmf[k] = term;
+    for (size_t k = 0; k + 1 < tail.size(); k++) {
         tail[k + 1] = std::max(0.0, tail[k] - term);
         term *= lambda / double(k + 1);
     }
-    double best = 1e300;
-    uint32_t w_best = 1;
-    for (uint32_t w = 1; w <= 4; w++) {
-        const double p = tail[2 * w];
-        double calls = 1.0;
-        for (int k = int(2 * w) + 2; k <= kMax && 32.0 * tail[k] > 0.5 * p; k += 2) calls += 1.0;
-        const double cost = 170.0 * w + 60.0 * (1.0 - std::pow(1.0 - p, 32.0)) + p * (300.0 + 230.0 * calls);
-        if (cost < best) {
-            best = cost;
-            w_best = w;
-            *left = p;
-        }
-    }
-    return w_best;
+}
+
+// Cost of a stream with a first window of w Philox calls (two draws each). A
+// walker runs the window for 32 streams at once and finishes the streams that
+// go on (2w or more events) 32 at a time, for as many calls as the longest of
+// the 32 needs. The terms (warp-instructions: a call of the window; setting
+// streams aside, when any of the 32 goes on; a finishing pass and each of its
+// calls) are fitted to the d=29 and d=11 surface-code workloads at windows of
+// 1 to 4 calls; at 4.1 expected events (p = 1e-3) windows of 2 / 3 / 4 calls
+// measured 491 / 296 / 310 ns per chunk, at 0.41 (p = 1e-4) windows of 1 / 2
+// calls 175 / 181.
+static double window_cost(const std::vector<double> &tail, uint32_t w) {
+    const double p = tail[2 * w];
+    double calls = 1.0;
+    for (size_t k = 2 * w + 2; k < tail.size() && 32.0 * tail[k] > 0.5 * p; k += 2) calls += 1.0;
+    return 170.0 * w + 60.0 * (1.0 - std::pow(1.0 - p, 32.0)) + p * (300.0 + 230.0 * calls);
 }
 
 // Share of a noise kind's drawn Pauli indices whose class is not 0.
@@ -163,6 +154,8 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
     G.compact_of.assign(G.noise.size(), 0xFFFFFFFFu);
     uint64_t slots = 0, long_lists = 0;
     uint32_t max_classes = 0;
+    std::vector<double> tail;
+    double cost[5] = {};
     for (uint32_t di = 0; di < G.noise.size(); di++) {
         const NoiseDesc &nd = G.noise[di];
         const uint32_t ng = sig_gens(nd.kind), KP = sig_paulis(nd.kind);
@@ -188,7 +181,11 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
                 it.lut |= uint64_t(cls[m]) << (4 * (k - 1));
             }
             const double lambda = 64.0 * double(u1 - u0) * table_p[nd.table];
-            it.calls = first_window_calls(lambda, &it.left);
+            poisson_tail(lambda, tail);
+            for (uint32_t w = 1; w <= 4; w++) {
+                cost[w] += window_cost(tail, w);
+                it.left[w] = tail[2 * w];
+            }
             it.events = lambda * live_share(nd, it.lut);
             max_classes = std::max(max_classes, it.classes);
             slots += uint64_t(u1 - u0) * it.classes;
@@ -201,6 +198,13 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
         }
     }
     G.n_compact_slots = slots;
+    // (the general kernel -- PAULI_CHANNEL_1 noise, more gap tables than
+    // shared memory holds next to a ring -- has windows of 1 and 3 only)
+    bool general = G.tables.size() / kTableWords > 4;
+    for (const NoiseDesc &nd : G.noise) general = general || nd.kind == N_PC1;
+    G.window_calls = 1;
+    for (uint32_t w = 2; w <= 4; w++)
+        if ((!general || w == 3) && cost[w] < cost[G.window_calls]) G.window_calls = w;
     // a list of three or more outputs costs the appliers a dependent read
     // of its own in the two-row layout: eight rows per slot when more than
     // one slot in sixteen has one (BB codes: about half; surface codes: a
@@ -810,7 +814,7 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
             for (uint32_t k = st.item_begin; k < st.item_end; k++) {
                 const CompactItem &ci = G.compact[G.compact_of[S.items[2 * k]] + S.items[2 * k + 1]];
                 ev += ci.events;
-                left += ci.left;
+                left += ci.left[G.window_calls];
             }
             S.step_events.push_back(float(ev));
             S.step_events.push_back(float(left));
@@ -828,7 +832,7 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
                 lut_words(G, ci, &lut_lo, &lut_hi);
                 const uint32_t w[8] = {uint32_t(m >> 32), uint32_t(m), sg, uint32_t(ci.slot0),
                                        nd.kind | (npauli << 3) | (ci.classes << 7) | ((units - 1) << 11) |
-                                           ((ci.calls - 1) << 17) | (nd.table << 19),
+                                           (nd.table << 19),
                                        lut_lo, lut_hi,
                                        G.tables[size_t(nd.table) * kTableWords + kGapLen]};
                 S.item_desc.insert(S.item_desc.end(), w, w + 8);

@@ -354,7 +354,7 @@ def tmcs_launch_shape(handle: int) -> Dict[str, object]:
     if name:
         extra = f", ring {w.value}" if w.value else ""
         if m.value == 7:
-            extra += f", {ap.value} applier warps" + (f", window {win.value}" if win.value else "")
+            extra += f", {ap.value} applier warps, window {win.value}"
         label = f"{name}<{k.value}> ({t.value} threads{extra})"
     return {"mode": m.value, "chunks": k.value, "threads": t.value, "ring_window": w.value, "kernel": label,
             "appliers": ap.value, "window": win.value, "global_arena": ga.value, "arena_entries": ae.value}
