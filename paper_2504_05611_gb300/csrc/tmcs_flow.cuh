@@ -34,9 +34,9 @@
 //
 // Measured (one GB300, 2070 MHz; before = one lane per stream with refills,
 // 8-byte event slots per Pauli index): d=29 non-local CNOT, p = 1e-3, 2e6
-// shots (12.39 GB of output): 11.2 ms before, 9.2 ms now (1.35 TB/s); the
-// same at p = 1e-4: 6.6, 5.1 (2.4 TB/s); d=11, 1e7 shots: 3.27, 2.78; BB144
-// teleport, 3e6: 3.02, 2.31. What bounds it now is the appliers' chain: a
+// shots (12.39 GB of output): 11.2 ms before, 9.2 ms now (1.34 TB/s); the
+// same at p = 1e-4: 6.6, 4.9 (2.5 TB/s); d=11, 1e7 shots: 3.28, 2.66; BB144
+// teleport, 3e6: 3.02, 2.06. What bounds it now is the appliers' chain: a
 // step of d=29 costs them 6.6 k cycles of application, 4.2 k of flush and 1.1 k
 // of waiting.
 #include <cuda.h>  // CUtensorMap (encoded through the runtime's driver entry point)
@@ -144,57 +144,59 @@ struct FlowLog {
     static constexpr uint32_t v = K == 1 ? 0 : K == 2 ? 1 : K == 4 ? 2 : K == 8 ? 3 : 4;
 };
 
-// One compact event slot as loaded: two rows per word (see SigSchedule::rows).
+// One compact event slot as loaded, two rows per word (see
+// SigSchedule::rows); the last word is two rows or the link to the next chunk
+// of a long list.
 template <bool WIDE>
 struct FlowSlot;
 template <>
 struct FlowSlot<false> {
-    uint32_t x;
-    __device__ __forceinline__ static FlowSlot load(const uint32_t *rows, uint32_t slot) { return {__ldg(rows + slot)}; }
+    uint32_t x, last;
+    __device__ __forceinline__ static FlowSlot load(const uint32_t *rows, uint32_t slot) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(rows) + slot);
+        return {v.x, v.y};
+    }
 };
 template <>
 struct FlowSlot<true> {
-    uint32_t x, y, z, w;
+    uint32_t x, y, z, last;
     __device__ __forceinline__ static FlowSlot load(const uint32_t *rows, uint32_t slot) {
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(rows) + slot);
         return {v.x, v.y, v.z, v.w};
     }
 };
 
-// XORs one event into the ring: word wv = event slot << (6 + log2 K) |
-// chunk << 6 | lane, v = the slot's rows.
+// XORs the rows of one loaded chunk into the ring for event word wv = event
+// slot << (6 + log2 K) | chunk << 6 | lane. Unused entries name the spare
+// row, so a pair is applied without tests; a word of two of them ends the
+// list.
 template <int K, bool WIDE>
 __device__ __forceinline__ void flow_put(const FlowArgs &A, uint64_t *ring, uint32_t wv, const FlowSlot<WIDE> &v) {
     // 32-bit word of the row that holds the event's lane: 2 chunk + lane / 32
     uint32_t *const base = reinterpret_cast<uint32_t *>(ring) + ((wv >> 5) & (2u * uint32_t(K) - 1u));
     const uint32_t bit = 1u << (wv & 31u);
-    auto put = [&](uint32_t row) { atomicXor(base + row * (2u * uint32_t(K)), bit); };
-    if (v.x & kRowOverflow) {
-        const uint32_t *ov = A.rows + (v.x & ~kRowOverflow);
-        const uint32_t n = __ldg(ov);
-        for (uint32_t i = 0; i < n; i += 2) {
-            const uint32_t w = __ldg(ov + 1 + i / 2);
-            put(w & 0xFFFFu);
-            put(w >> 16);
-        }
-        return;
-    }
-    // unused entries of a word name the spare row
-    put(v.x & 0xFFFFu);
-    put(v.x >> 16);
+    const uint32_t spare = (A.window_mask + 1u + A.n_obs) * 0x10001u;
+    auto pair = [&](uint32_t w) {
+        atomicXor(base + (w & 0xFFFFu) * (2u * uint32_t(K)), bit);
+        atomicXor(base + (w >> 16) * (2u * uint32_t(K)), bit);
+    };
+    pair(v.x);
     if constexpr (WIDE) {
-        // a word whose first entry is the spare row holds nothing, nor do
-        // those after it
-        const uint32_t spare = A.window_mask + 1u + A.n_obs;
-        if ((v.y & 0xFFFFu) == spare) return;
-        put(v.y & 0xFFFFu);
-        put(v.y >> 16);
-        if ((v.z & 0xFFFFu) == spare) return;
-        put(v.z & 0xFFFFu);
-        put(v.z >> 16);
-        if ((v.w & 0xFFFFu) == spare) return;
-        put(v.w & 0xFFFFu);
-        put(v.w >> 16);
+        if (v.y == spare) return;
+        pair(v.y);
+        if (v.z == spare) return;
+        pair(v.z);
+    }
+    if (v.last != spare && !(v.last & kRowOverflow)) pair(v.last);
+}
+
+// One event from its slot on, chunk by chunk.
+template <int K, bool WIDE>
+__device__ __forceinline__ void flow_put_all(const FlowArgs &A, uint64_t *ring, uint32_t wv, FlowSlot<WIDE> v) {
+    for (;;) {
+        flow_put<K, WIDE>(A, ring, wv, v);
+        if (!(v.last & kRowOverflow)) return;
+        v = FlowSlot<WIDE>::load(A.rows, v.last & ~kRowOverflow);
     }
 }
 
@@ -294,7 +296,7 @@ struct FlowWalker {
         s.kpm = (((d1.x >> 7) & 15u) << S_EV) - 64u;
         s.tab1 = (d1.x >> 19) * kTableWords - 1u;
         s.desc = d1.z;
-        // two-row layout: 30 bits, kept S_EV bits up so that the shift by a
+        // four-row layout: 30 bits, kept S_EV bits up so that the shift by a
         // Pauli index leaves its class in place in the event word
         s.lut = WIDE ? uint64_t(d1.y) | (uint64_t(d1.z) << 32) : uint64_t(d1.y) << S_EV;
         s.inv = __uint_as_float(d1.w);
@@ -339,7 +341,7 @@ struct FlowWalker {
             }
             __nanosleep(64);
         }
-        flow_put<K, WIDE>(A, ring, wv, FlowSlot<WIDE>::load(A.rows, wv >> S_EV));
+        flow_put_all<K, WIDE>(A, ring, wv, FlowSlot<WIDE>::load(A.rows, wv >> S_EV));
     }
 
     // Stores the lane's events of a window (those with live[d]) in the step's
@@ -583,16 +585,6 @@ __device__ __forceinline__ void tma_commit() { asm volatile("cp.async.bulk.commi
 __device__ __forceinline__ void tma_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// Flush of detectors [z, w) with tensor stores: the rows of each ring
-// segment (at most two: the ring wraps) go out as boxes of tma_rows rows x K
-// chunk words issued by the first applier warp, starting at a ring row whose
-// address is 128-byte aligned; the few rows before that point and after the
-// last whole box are written with plain stores. Every row is cleared: the
-// boxes' rows once the tensor stores have read them. The last column of the
-// call (in the call's last tile) gets its pad bits masked in the ring first.
-// Every applier has fenced its ring writes for the async proxy before the
-// barrier that precedes this call. Ends with the boxes' rows cleared; the
-// caller's barrier follows.
 // Rows [d0, d1) of one contiguous stretch of the ring: plain head rows
 // [d0, dh) up to the first 128-byte aligned ring row, whole boxes [dh, db),
 // plain tail rows [db, d1).
@@ -737,33 +729,42 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
             __threadfence_block();  // the walkers' events precede the reads below
             const uint32_t cap = S.scap[q];
             const uint32_t n = min(ld_shared_volatile(&C.cnt[slot]), cap);
-            // whole batches first: no bounds in the loop but the wrap
+            // Batches of kFlowApplyBatch events per thread: their slot loads
+            // overlap, then their rows are applied, then the next chunks of
+            // those with long lists are loaded together, and so on. (Each
+            // event's list followed to its end before the next event cost a
+            // dependent L2 read per event: with two rows per slot 2 % of the
+            // events of a surface code had one, so half of all warp-wide
+            // events did.)
             const uint32_t per = nthr * kFlowApplyBatch;
-            uint32_t e = at;
             auto entry = [&](uint32_t i) {
                 const uint32_t a = up + i;
                 return arena[a >= A.arena ? a - A.arena : a];
             };
-            for (; e + (per - nthr) < n; e += per) {
-                uint32_t wv[kFlowApplyBatch];
-                FlowSlot<WIDE> v[kFlowApplyBatch];
-#pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++) wv[j] = entry(e + j * nthr);
-#pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++) v[j] = FlowSlot<WIDE>::load(A.rows, wv[j] >> S_EV);
-#pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++) flow_put<K, WIDE>(A, S.ring, wv[j], v[j]);
-            }
-            if (e < n) {  // the rest, its loads still overlapped
+            for (uint32_t e = at; e < n; e += per) {
                 uint32_t wv[kFlowApplyBatch];
                 FlowSlot<WIDE> v[kFlowApplyBatch];
 #pragma unroll
                 for (uint32_t j = 0; j < kFlowApplyBatch; j++) wv[j] = entry(min(e + j * nthr, n - 1u));
 #pragma unroll
                 for (uint32_t j = 0; j < kFlowApplyBatch; j++) v[j] = FlowSlot<WIDE>::load(A.rows, wv[j] >> S_EV);
+                uint32_t go = 0;  // bit j: event j has a chunk to apply
 #pragma unroll
-                for (uint32_t j = 0; j < kFlowApplyBatch; j++)
-                    if (e + j * nthr < n) flow_put<K, WIDE>(A, S.ring, wv[j], v[j]);
+                for (uint32_t j = 0; j < kFlowApplyBatch; j++) go |= e + j * nthr < n ? 1u << j : 0u;
+                for (;;) {
+                    uint32_t more = 0;
+#pragma unroll
+                    for (uint32_t j = 0; j < kFlowApplyBatch; j++)
+                        if ((go >> j) & 1u) {
+                            flow_put<K, WIDE>(A, S.ring, wv[j], v[j]);
+                            more |= (v[j].last >> 31) << j;
+                        }
+                    if (!more) break;
+                    go = more;
+#pragma unroll
+                    for (uint32_t j = 0; j < kFlowApplyBatch; j++)
+                        if ((go >> j) & 1u) v[j] = FlowSlot<WIDE>::load(A.rows, v[j].last & ~kRowOverflow);
+                }
             }
             if (tma) fence_proxy_async_shared();  // ring writes before the tensor stores read them
             flow_bar(nthr);

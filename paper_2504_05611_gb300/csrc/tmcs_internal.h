@@ -214,7 +214,7 @@ struct SigSchedule {
     // round 1), segment, first compact event slot, kind | npauli << 3 |
     // classes per unit << 7 | (units - 1) << 11 | table << 19, then the class of every Pauli index as nibbles
     // (index k at bit 4 (k - 1) of the 64-bit word 5 | word 6 << 32; 0 = it
-    // flips nothing in any unit of the segment; in the two-row layout, where
+    // flips nothing in any unit of the segment; in the four-row layout, where
     // no segment has more than three classes, two bits per index in word 5;
     // PAULI_CHANNEL_1 has three indices, and its descriptor index in word
     // 6), and the float bits of 1/log2(1-p) (the gap estimate).
@@ -222,10 +222,10 @@ struct SigSchedule {
     // Output lists of the compact event slots as rows of this schedule's
     // ring (barrier schedules): row = detector mod window, or window +
     // observable; unused entries name a spare row, window + observables,
-    // that nothing reads. A slot is one word of two 16-bit rows, or four
-    // words of eight (SigProgram::wide); bit 31 of the first word marks a
-    // longer list: kRowOverflow | word offset of a list [count, rows two per
-    // word] after the slots.
+    // that nothing reads. A slot is a chunk of four 16-bit rows (two words),
+    // or of eight (SigProgram::wide); a list that does not fit has its last
+    // word replaced by kRowOverflow | index of the chunk that goes on with it
+    // (chunks after the slots, counted from the table's start).
     std::vector<uint32_t> rows;
 };
 
@@ -274,7 +274,7 @@ struct SigProgram {
     std::vector<uint32_t> compact_of;  // first CompactItem index of each descriptor's segments (0xFFFFFFFF: none)
     uint64_t n_compact_slots = 0;
     uint32_t window_calls = 1;         // Philox calls of a stream's first window in the decoupled kernel
-    bool wide = false;                 // eight rows per slot instead of two, up to 15 classes instead of 3
+    bool wide = false;                 // eight rows per slot instead of four, up to 15 classes instead of 3
     double build_seconds = 0;
 };
 

@@ -94,7 +94,7 @@ static void event_list(const SigProgram &G, size_t k, std::vector<uint32_t> &v) 
 }
 
 // Words of a compact event slot.
-static size_t slot_words(const SigProgram &G) { return G.wide ? 4 : 1; }
+static size_t slot_words(const SigProgram &G) { return G.wide ? 4 : 2; }
 
 // Distribution of a stream's events (Poisson with mean lambda): P(X >= k).
 static void poisson_tail(double lambda, std::vector<double> &tail) {
@@ -192,7 +192,8 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
             for (uint32_t u = u0; u < u1; u++)
                 for (uint32_t c = 1; c <= it.classes; c++) {
                     const size_t k = G.ev_base[di] + size_t(u) * KP + (it.rep[c] - 1u);
-                    if (G.ev_ent[2 * k] != kEvNone && (G.ev_ent[2 * k] & kEvOverflow)) long_lists++;
+                    if (G.ev_ent[2 * k] != kEvNone && (G.ev_ent[2 * k] & kEvOverflow) && G.ev_ent[2 * k + 1] > 4)
+                        long_lists++;
                 }
             G.compact.push_back(it);
         }
@@ -205,11 +206,12 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
     G.window_calls = 1;
     for (uint32_t w = 2; w <= 4; w++)
         if ((!general || w == 3) && cost[w] < cost[G.window_calls]) G.window_calls = w;
-    // a list of three or more outputs costs the appliers a dependent read
-    // of its own in the two-row layout: eight rows per slot when more than
-    // one slot in sixteen has one (BB codes: about half; surface codes: a
-    // few per cent), or when a segment has more classes than its layout holds
-    G.wide = long_lists * 16 > slots || max_classes > 3;
+    // a list that does not fit its slot costs the appliers a dependent read:
+    // eight rows per slot when more than one list in 500 has more than four
+    // (BB codes: about half; surface codes: none), so that a warp's 128
+    // events of a batch seldom hold one; also when a segment has more
+    // classes than the four-row layout holds
+    G.wide = long_lists * 500 > slots || max_classes > 3;
 }
 
 static uint32_t row_of(uint32_t entry, uint32_t W) {
@@ -231,19 +233,22 @@ static bool build_rows(const SigProgram &G, uint64_t O, SigSchedule &S) {
         for (uint32_t u = 0; u < units; u++)
             for (uint32_t c = 1; c <= it.classes; c++) {
                 event_list(G, G.ev_base[it.desc] + size_t(u0 + u) * KP + (it.rep[c] - 1u), v);
-                const size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr;
+                size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr;
                 for (uint32_t &e : v) e = row_of(e, S.window);
-                size_t to = at;
-                if (v.size() > 2 * wpr) {
-                    to = S.rows.size() + 1;
-                    if (to + v.size() / 2 + 1 >= (uint64_t(1) << 31)) return false;
-                    S.rows[at] = kRowOverflow | uint32_t(S.rows.size());
-                    S.rows.push_back(uint32_t(v.size()));
-                    S.rows.resize(S.rows.size() + (v.size() + 1) / 2, none);
-                }
-                for (size_t x = 0; x < v.size(); x++) {
-                    uint32_t &w = S.rows[to + x / 2];
-                    w = (x & 1) ? (w & 0xFFFFu) | (v[x] << 16) : (w & 0xFFFF0000u) | v[x];
+                // chunks: all rows, or all but two and a link
+                for (size_t x = 0; x < v.size();) {
+                    const bool link = v.size() - x > 2 * wpr;
+                    const size_t n = link ? 2 * wpr - 2 : v.size() - x;
+                    for (size_t i = 0; i < n; i++, x++) {
+                        uint32_t &w = S.rows[at + i / 2];
+                        w = (i & 1) ? (w & 0xFFFFu) | (v[x] << 16) : (w & 0xFFFF0000u) | v[x];
+                    }
+                    if (!link) break;
+                    const size_t chunk = S.rows.size() / wpr;
+                    if (chunk >= (uint64_t(1) << 31)) return false;
+                    S.rows[at + wpr - 1] = kRowOverflow | uint32_t(chunk);
+                    at = S.rows.size();
+                    S.rows.resize(S.rows.size() + wpr, none);
                 }
             }
     }
@@ -258,7 +263,7 @@ static std::string validate_rows(const SigProgram &G, uint64_t O, const SigSched
     const size_t wpr = slot_words(G);
     if (S.rows.size() < G.n_compact_slots * wpr || uint64_t(S.window) + O >= 0x7FFFu) return "row table size";
     const uint32_t spare = S.window + uint32_t(O);
-    std::vector<uint32_t> v, r, prev;
+    std::vector<uint32_t> v;
     for (const CompactItem &it : G.compact) {
         const NoiseDesc &nd = G.noise[it.desc];
         const uint32_t KP = sig_paulis(nd.kind);
@@ -274,24 +279,22 @@ static std::string validate_rows(const SigProgram &G, uint64_t O, const SigSched
                     continue;
                 }
                 event_list(G, ek, v);
-                const uint32_t *w = &S.rows[(it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr];
-                size_t n = 2 * wpr;
-                if (w[0] & kRowOverflow) {
-                    const size_t off = w[0] & ~kRowOverflow;
-                    if (off < G.n_compact_slots * wpr || off >= S.rows.size()) return "row list";
-                    n = S.rows[off];
-                    w = S.rows.data() + off + 1;
-                    if (n <= 2 * wpr || off + 1 + (n + 1) / 2 > S.rows.size()) return "row list";
+                size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr, x = 0;
+                for (;;) {
+                    const uint32_t last = S.rows[at + wpr - 1];
+                    const bool link = (last & kRowOverflow) != 0;
+                    if (link != (v.size() - x > 2 * wpr)) return "row list";
+                    const size_t n = link ? 2 * wpr - 2 : 2 * wpr;
+                    for (size_t i = 0; i < n; i++) {
+                        const uint32_t row = (S.rows[at + i / 2] >> (16 * (i & 1))) & 0xFFFFu;
+                        // entries past the list name the spare row
+                        if (row != (x < v.size() ? row_of(v[x], S.window) : spare)) return "event row";
+                        if (x < v.size()) x++;
+                    }
+                    if (!link) break;
+                    at = size_t(last & ~kRowOverflow) * wpr;
+                    if (at < G.n_compact_slots * wpr || at + wpr > S.rows.size()) return "row list";
                 }
-                size_t x = 0;
-                for (; x < n; x++) {
-                    const uint32_t row = (w[x / 2] >> (16 * (x & 1))) & 0xFFFFu;
-                    if (row == spare) break;
-                    if (x >= v.size() || row != row_of(v[x], S.window)) return "event row";
-                }
-                if (x != v.size()) return "event row";
-                for (; x < n + (n & 1); x++)  // the rest names the spare row
-                    if (((w[x / 2] >> (16 * (x & 1))) & 0xFFFFu) != spare) return "event row";
             }
     }
     return std::string();

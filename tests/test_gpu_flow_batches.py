@@ -6,7 +6,7 @@ Philox calls and puts the streams that go on aside in blocks of 32 (Methods
 sit at the edges: windows so short that nearly every stream goes on, blocks
 that fill and overflow the step's space for them, steps whose items do not
 fill a batch, chunk counts that do not fill a tile, and both slot layouts
-(two rows per event, and eight for codes whose events flip many outputs).
+(four rows per event, and eight for codes whose events flip many outputs).
 The outputs are bits: they must equal the oracle's.
 """
 import numpy as np
