@@ -22,8 +22,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libtmcs.so")
 SOURCES = ["tmcs_host.cpp", "tmcs_signature.cpp", "tmcs_sample.cu", "tmcs_flow.cu", "tmcs_flow_k1.cu",
-           "tmcs_flow_k2.cu", "tmcs_flow_k4.cu", "tmcs_flow_k8.cu", "tmcs_flow_k16.cu", "tmcs_server.cu",
-           "tmcs_peaks.cu"]
+           "tmcs_flow_k2.cu", "tmcs_flow_k4.cu", "tmcs_flow_k8.cu", "tmcs_flow_k16.cu", "tmcs_flow_batch.cu",
+           "tmcs_server.cu", "tmcs_peaks.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

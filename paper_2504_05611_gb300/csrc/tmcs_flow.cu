@@ -28,7 +28,7 @@ bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int applie
     if (!G.ok || sched < 0 || size_t(sched) >= G.sched.size()) return false;
     const SigSchedule &S = G.sched[sched];
     if (S.lag || S.rows.empty() || S.steps.empty() || S.steps.size() > kFlowMaxSteps ||
-        S.step_events.size() != 2 * S.steps.size())
+        S.step_events.size() != 5 * S.steps.size())
         return false;
     if (K != 1 && K != 2 && K != 4 && K != 8 && K != 16) return false;
     if (threads < 64 || threads > TMCS_FLOW_MAX_THREADS || threads % 32 || appliers < 1 || appliers >= threads / 32)
@@ -104,17 +104,17 @@ static bool encode_det_map(CUtensorMap *map, uint64_t *det, uint64_t n_det, uint
            CUDA_SUCCESS;
 }
 
-cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
-                        const FlowCall &call, int sms, cudaStream_t st) {
-    if (!ds || s.sched < 0 || size_t(s.sched) >= G.sched.size() || !ds->rows[s.sched])
-        return cudaErrorInvalidValue;
+// What a launch of this shape takes from the program and the call, without
+// the columns.
+static FlowArgs flow_args(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
+                          const FlowCall &call) {
     const SigSchedule &S = G.sched[s.sched];
     FlowArgs a{};
     a.noise = ds->noise;
     a.tables = ds->tables;
     a.item_desc = reinterpret_cast<const uint4 *>(ds->item_desc[s.sched]);
     a.steps = reinterpret_cast<const uint4 *>(ds->steps[s.sched]);
-    a.step_events = reinterpret_cast<const float2 *>(ds->step_events[s.sched]);
+    a.step_events = ds->step_events[s.sched];
     a.rows = ds->rows[s.sched];
     a.n_steps = uint32_t(S.steps.size());
     a.window_mask = S.window - 1u;
@@ -135,6 +135,94 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     a.key1 = call.key1;
     a.keys = philox_keys(call.key0, call.key1);
     a.ld = call.n_cols;
+    a.status = call.status;
+    return a;
+}
+
+// Columns [c0, c0 + n) of the call.
+static void flow_columns(FlowArgs &a, const FlowShape &s, const FlowCall &call, uint64_t c0, uint64_t n) {
+    a.first_chunk = call.first_chunk + uint32_t(c0);
+    a.n_cols = n;
+    a.last_mask = c0 + n == call.n_cols ? call.last_mask : ~uint64_t(0);
+    a.n_tiles = (n + uint64_t(s.K) - 1) / uint64_t(s.K);
+    a.det = call.det + c0;
+    a.col_base = c0;
+    a.obs = call.obs ? call.obs + c0 : nullptr;
+    a.vec_out = (reinterpret_cast<uintptr_t>(a.det) % 16 == 0 && a.ld % 2 == 0) ? 1u : 0u;
+}
+
+static uint64_t batches_per_tile(const SigSchedule &S, int K) {
+    const uint64_t ipb = 32u / uint64_t(K);
+    uint64_t n = 0;
+    for (const SigStep &t : S.steps) n += (t.item_end - t.item_begin + ipb - 1) / ipb;
+    return n;
+}
+
+int flow_batch_tile() { return kFlowBatchK; }
+
+cudaError_t flow_batch(const std::vector<FlowJob> &jobs, int sms, cudaStream_t st) {
+    struct Entry {
+        const FlowJob *j;
+        FlowArgs a;
+        double tile;  // relative time of a tile
+    };
+    // one launch per kernel variant (and per kFlowBatchJobs jobs)
+    for (int variant = 0; variant < 4; variant++) {
+        const bool wide = (variant & 1) != 0, fast = (variant & 2) != 0;
+        std::vector<Entry> v;
+        int window = 1;
+        for (const FlowJob &j : jobs) {
+            const SigProgram &G = j.c->sig;
+            Entry e{&j, flow_args(G, uint32_t(j.c->n_obs), j.ds, j.shape, j.call), 0.0};
+            if (G.wide != wide || (e.a.smem_tables && e.a.near && !e.a.pc1) != fast) continue;
+            flow_columns(e.a, j.shape, j.call, 0, j.call.n_cols);
+            // batches, events and detectors of a tile, in walker-instruction
+            // terms, and the steps' hand-overs
+            const SigSchedule &S = G.sched[j.shape.sched];
+            double events = 0;
+            for (size_t k = 0; k < S.step_events.size(); k += 5) events += double(S.step_events[k]);
+            e.tile = 600.0 * double(batches_per_tile(S, kFlowBatchK)) +
+                     kFlowBatchK * (2.0 * events + 1.0 * double(G.n_det)) + 2000.0 * double(S.steps.size());
+            window = std::max(window, int(G.window_calls));
+            v.push_back(e);
+        }
+        for (size_t base = 0; base < v.size(); base += kFlowBatchJobs) {
+            const size_t n = std::min<size_t>(kFlowBatchJobs, v.size() - base);
+            // CTAs: one each, then one more for the job that would finish
+            // last, until every SM has one
+            std::vector<uint32_t> ctas(n, 1);
+            auto time = [&](size_t i, uint32_t c) {
+                const Entry &e = v[base + i];
+                return double((e.a.n_tiles + c - 1) / c) * e.tile;
+            };
+            for (uint32_t used = uint32_t(n); used < uint32_t(sms); used++) {
+                size_t worst = 0;
+                for (size_t i = 1; i < n; i++)
+                    if (time(i, ctas[i]) > time(worst, ctas[worst])) worst = i;
+                if (ctas[worst] >= v[base + worst].a.n_tiles) break;
+                ctas[worst]++;
+            }
+            FlowBatchArgs b;
+            std::memset(static_cast<void *>(&b), 0, sizeof(b));
+            size_t smem = 0;
+            for (size_t i = 0; i < n; i++) {
+                b.jobs[i] = v[base + i].a;
+                b.cta_begin[i + 1] = b.cta_begin[i] + ctas[i];
+                smem = std::max(smem, v[base + i].j->shape.smem);
+            }
+            b.n_jobs = uint32_t(n);
+            const cudaError_t e = flow_batch_launch(b, wide, fast, window, v[base].j->shape.threads, smem, st);
+            if (e != cudaSuccess) return e;
+        }
+    }
+    return cudaSuccess;
+}
+
+cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
+                        const FlowCall &call, int sms, cudaStream_t st) {
+    if (!ds || s.sched < 0 || size_t(s.sched) >= G.sched.size() || !ds->rows[s.sched]) return cudaErrorInvalidValue;
+    const SigSchedule &S = G.sched[s.sched];
+    FlowArgs a = flow_args(G, n_obs, ds, s, call);
     // tensor-store flush: by default for tiles of 8 or more chunks (rows of
     // 64 bytes or more; narrower boxes measured slower than plain stores);
     // TMCS_FLOW_TMA=1 for any even tile, 0 never; TMCS_FLOW_TMA_ROWS sets
@@ -148,9 +236,7 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     // A CTA counts its batches and its steps in 32 bits: a call with more
     // tiles per CTA than that allows runs as several launches over column
     // slices (each a multiple of the tile size, in column order).
-    const uint64_t ipb = 32u / uint64_t(s.K);
-    uint64_t per_tile_batches = 0;
-    for (const SigStep &t : S.steps) per_tile_batches += (t.item_end - t.item_begin + ipb - 1) / ipb;
+    const uint64_t per_tile_batches = batches_per_tile(S, s.K);
     const uint64_t per_tile_steps = a.n_steps;
     const uint64_t lim = (uint64_t(1) << 31) - 1;
     const uint64_t max_tiles_per_cta =
@@ -162,15 +248,7 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     if (tslice > 0) slice_cols = std::min<uint64_t>(slice_cols, uint64_t(tslice) * uint64_t(s.K));
     for (uint64_t c0 = 0; c0 < call.n_cols; c0 += slice_cols) {
         const uint64_t n = std::min(slice_cols, call.n_cols - c0);
-        a.first_chunk = call.first_chunk + uint32_t(c0);
-        a.n_cols = n;
-        a.last_mask = c0 + n == call.n_cols ? call.last_mask : ~uint64_t(0);
-        a.n_tiles = (n + uint64_t(s.K) - 1) / uint64_t(s.K);
-        a.det = call.det + c0;
-        a.col_base = c0;
-        a.obs = call.obs ? call.obs + c0 : nullptr;
-        a.vec_out = (reinterpret_cast<uintptr_t>(a.det) % 16 == 0 && a.ld % 2 == 0) ? 1u : 0u;
-        a.status = call.status;
+        flow_columns(a, s, call, c0, n);
         const bool fast = a.smem_tables && a.near && !a.pc1;
         cudaError_t e;
         switch (s.K) {

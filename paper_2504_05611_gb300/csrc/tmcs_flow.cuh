@@ -66,7 +66,7 @@ struct FlowArgs {
     const uint32_t *tables;
     const uint4 *item_desc;     // walker descriptors, two uint4 per item (see SigSchedule::item_desc)
     const uint4 *steps;         // item_begin, item_end, flush_lo, flush_hi
-    const float2 *step_events;  // expected live events and unfinished streams per chunk of each step
+    const float *step_events;   // per step: expected live events, unfinished streams by window (SigSchedule)
     const uint32_t *rows;       // ring rows of every compact event slot (see SigSchedule::rows)
     uint32_t n_steps, window_mask, n_obs;
     uint32_t arena;             // arena entries
@@ -271,6 +271,7 @@ struct FlowWalker {
     FlowCtl &C;
     const uint32_t *tabs;
     uint32_t lane, lt;
+    uint32_t bx, gx;  // the CTA among those of its job, their number
     // the step being walked: sequence number, first item, item end, batches,
     // region (position in the arena, capacity for events and for put-aside
     // streams), tile's first chunk, valid chunks
@@ -530,7 +531,7 @@ struct FlowWalker {
                 lcap = S.slcap[q];
                 const uint32_t U = T * c_tile + S.soff[q];  // modulo 2^32
                 upos = uint32_t((uint64_t(T) * c_tile + S.soff[q]) % A.arena);
-                chunk0 = A.first_chunk + (blockIdx.x + T * gridDim.x) * uint32_t(K);
+                chunk0 = A.first_chunk + (bx + T * gx) * uint32_t(K);
                 nv = T == nt - 1u ? nv_last : uint32_t(K);
                 if (!wait_gate(U + cap + lcap - A.arena)) return;
             }
@@ -668,7 +669,7 @@ __device__ __forceinline__ void flow_flush_tma(const FlowArgs &A, const FlowSmem
 // Applier warps: steps in CTA order.
 template <int K, bool WIDE>
 __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S, FlowCtl &C, uint32_t nt,
-                                           uint32_t nv_last) {
+                                           uint32_t nv_last, uint32_t bx, uint32_t gx) {
     constexpr uint32_t LK = FlowLog<K>::v, S_EV = 6u + LK;
     const uint32_t nthr = blockDim.x - 32u * A.walkers;
     const uint32_t at = threadIdx.x - 32u * A.walkers;
@@ -683,7 +684,7 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
     uint32_t U = 0;   // arena position of step Q, modulo 2^32
     uint32_t up = 0;  // the same modulo the arena size
     for (uint32_t T = 0; T < nt; T++) {
-        const uint64_t tile = uint64_t(blockIdx.x) + uint64_t(T) * gridDim.x;
+        const uint64_t tile = uint64_t(bx) + uint64_t(T) * gx;
         const uint64_t col0 = tile * uint64_t(K);
         const uint32_t nv = T == nt - 1u ? nv_last : uint32_t(K);
         for (uint32_t q = 0; q < A.n_steps; q++) {
@@ -847,11 +848,10 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
 #define TMCS_FLOW_MAX_THREADS 1024
 #endif
 
+// One CTA (number bx of gx) of a job: tiles bx, bx + gx, ...
 template <int K, bool WIDE, bool FAST, int W>
-__global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __grid_constant__ FlowArgs A) {
-    extern __shared__ __align__(128) uint64_t smem[];
-    __shared__ FlowCtl C;
-    if (uint64_t(blockIdx.x) >= A.n_tiles) return;
+__device__ __forceinline__ void flow_cta(const FlowArgs &A, uint64_t *smem, FlowCtl &C, uint32_t bx, uint32_t gx) {
+    if (uint64_t(bx) >= A.n_tiles) return;
     const FlowSmem S = flow_layout(smem, A, K);
     const uint32_t tid = threadIdx.x, T_ = blockDim.x;
     const uint32_t rows = A.window_mask + 1u;
@@ -862,8 +862,7 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
     // hold none
     for (uint32_t i = tid; i < A.n_steps; i += T_) {
         const uint4 st = __ldg(A.steps + i);
-        const float2 ex = __ldg(A.step_events + i);
-        const float mu = ex.x * float(K), ml = ex.y * float(K);
+        const float mu = __ldg(A.step_events + 5 * i) * float(K), ml = __ldg(A.step_events + 5 * i + W) * float(K);
         uint32_t cap = A.test_cap ? A.test_cap : uint32_t(ceilf(mu + 6.0f * sqrtf(mu) + 64.0f));
         // put-aside streams: whole blocks, at most a quarter of the arena
         uint32_t lcap = min((uint32_t(ceilf(ml + 6.0f * sqrtf(ml))) + 63u) & ~31u, (A.arena / 4u) & ~31u);
@@ -912,20 +911,68 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
         }
         if (!bat && l == 31) S.soff[A.n_steps] = incl;
     }
-    const uint64_t G = gridDim.x;
-    const uint32_t nt = uint32_t((A.n_tiles - blockIdx.x + G - 1) / G);
-    const uint64_t last = uint64_t(blockIdx.x) + uint64_t(nt - 1) * G;
+    const uint32_t nt = uint32_t((A.n_tiles - bx + gx - 1) / gx);
+    const uint64_t last = uint64_t(bx) + uint64_t(nt - 1) * gx;
     const uint64_t rem = A.n_cols - last * K;
     const uint32_t nv_last = rem < uint64_t(K) ? uint32_t(rem) : uint32_t(K);
     __syncthreads();
     if ((tid >> 5) >= A.walkers) {
-        flow_apply<K, WIDE>(A, S, C, nt, nv_last);
+        flow_apply<K, WIDE>(A, S, C, nt, nv_last, bx, gx);
     } else {
         const uint32_t lane = tid & 31u;
-        FlowWalker<K, FAST, WIDE, W> w{A, S, C, FAST ? S.stab : A.tables, lane, (1u << lane) - 1u};
+        FlowWalker<K, FAST, WIDE, W> w{A, S, C, FAST ? S.stab : A.tables, lane, (1u << lane) - 1u, bx, gx};
         w.run(nt, nv_last);
     }
 }
+
+template <int K, bool WIDE, bool FAST, int W>
+__global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __grid_constant__ FlowArgs A) {
+    extern __shared__ __align__(128) uint64_t smem[];
+    __shared__ FlowCtl C;
+    flow_cta<K, WIDE, FAST, W>(A, smem, C, blockIdx.x, gridDim.x);
+}
+
+// Many small circuits in one launch: every CTA works on one job, and a job
+// has as many CTAs as its share of the work (the host's choice), so the jobs
+// run side by side and none waits for a launch of its own. The job table is
+// a kernel parameter, so a graph can hold the launch. Tiles of four chunks:
+// the jobs are those that do not fill the GPU alone.
+constexpr int kFlowBatchK = 4;
+constexpr uint32_t kFlowBatchJobs = 64;
+struct FlowBatchArgs {
+    FlowArgs jobs[kFlowBatchJobs];
+    uint32_t cta_begin[kFlowBatchJobs + 1];  // first CTA of each job; [n_jobs] = all
+    uint32_t n_jobs;
+};
+static_assert(sizeof(FlowBatchArgs) <= 32000, "the job table exceeds the kernel parameter limit");
+
+template <bool WIDE, bool FAST, int W>
+__global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_batch_kernel(const __grid_constant__ FlowBatchArgs B) {
+    extern __shared__ __align__(128) uint64_t smem[];
+    __shared__ FlowCtl C;
+    uint32_t lo = 0, hi = B.n_jobs - 1u;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1u) / 2u;
+        if (B.cta_begin[mid] <= blockIdx.x) lo = mid;
+        else hi = mid - 1u;
+    }
+    flow_cta<kFlowBatchK, WIDE, FAST, W>(B.jobs[lo], smem, C, blockIdx.x - B.cta_begin[lo],
+                                         B.cta_begin[lo + 1u] - B.cta_begin[lo]);
+}
+
+template <bool WIDE, bool FAST, int W>
+cudaError_t flow_batch_go(const FlowBatchArgs &b, int threads, size_t smem, cudaStream_t st) {
+    auto kern = flow_batch_kernel<WIDE, FAST, W>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
+    if (e != cudaSuccess) return e;
+    kern<<<b.cta_begin[b.n_jobs], threads, smem, st>>>(b);
+    return cudaGetLastError();
+}
+// Dispatch over its variants (tmcs_flow_batch.cu).
+cudaError_t flow_batch_launch(const FlowBatchArgs &b, bool wide, bool fast, int window, int threads, size_t smem,
+                              cudaStream_t st);
 
 // Launch of one kernel variant: a persistent grid of the CTAs that are
 // resident at once, never more than there are tiles.

@@ -204,10 +204,10 @@ struct SigSchedule {
     // (units - 1) << 16 | descriptor << 22 (descriptor < 1024, table < 8192).
     std::vector<uint32_t> item_rec;
     std::vector<SigStep> steps;
-    // Two numbers per step, expected per 64-shot chunk: the events that flip
+    // Five numbers per step, expected per 64-shot chunk: the events that flip
     // something (sum over its items of 64 x units x p x live share), and the
-    // streams that do not end in their first window; the decoupled kernel
-    // sizes the step's arena region by them.
+    // streams that do not end in a first window of 1, 2, 3, 4 calls; the
+    // decoupled kernel sizes the step's arena region by them.
     std::vector<float> step_events;
     // Walker descriptors of the decoupled kernel, 8 words per item (no
     // dependence on the seed): hi and lo of 0xCD9E8D57 x op index (Philox
@@ -351,6 +351,16 @@ void free_device_programs(tmcs_circuit *c);
 // the given schedule, chunks per tile, CTA size and applier warps if that shape fits `budget` bytes of dynamic shared memory.
 bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out);
 #ifdef __CUDACC__
+// One circuit of a batched launch of the decoupled kernel.
+struct FlowJob {
+    const tmcs_circuit *c = nullptr;
+    const DeviceSig *ds = nullptr;
+    FlowShape shape;   // tiles of flow_batch_tile() chunks
+    FlowCall call;
+};
+int flow_batch_tile();
+// Runs all jobs in as few launches as their kernel variants allow.
+cudaError_t flow_batch(const std::vector<FlowJob> &jobs, int sms, cudaStream_t st);
 cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
                         const FlowCall &call, int sms, cudaStream_t st);
 #endif

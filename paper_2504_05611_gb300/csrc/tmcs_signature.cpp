@@ -368,7 +368,7 @@ static std::string validate_signature_program(const SigProgram &G, uint64_t D, u
         const uint32_t W = S.window;
         if (W < 256 || (W & (W - 1)) || S.lag > uint32_t(kSigMaxLag) || (S.lag && W > 16384)) return "schedule shape";
         if (S.item_rec.size() != 4 * n_items || S.steps.empty()) return "schedule size";
-        if (S.step_events.size() != 2 * S.steps.size()) return "step event counts";
+        if (S.step_events.size() != 5 * S.steps.size()) return "step event counts";
         if (S.item_desc.size() != 8 * n_items || S.steps.size() > (1u << 15)) return "walker descriptors size";
         std::vector<uint64_t> lo(n_items), hi(n_items);
         for (size_t k = 0; k < n_items; k++) {
@@ -813,14 +813,14 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
         }
         // expected live events and unfinished streams per chunk of each step
         for (const SigStep &st : S.steps) {
-            double ev = 0, left = 0;
+            double ev = 0, left[5] = {};
             for (uint32_t k = st.item_begin; k < st.item_end; k++) {
                 const CompactItem &ci = G.compact[G.compact_of[S.items[2 * k]] + S.items[2 * k + 1]];
                 ev += ci.events;
-                left += ci.left[G.window_calls];
+                for (uint32_t w = 1; w <= 4; w++) left[w] += ci.left[w];
             }
             S.step_events.push_back(float(ev));
-            S.step_events.push_back(float(left));
+            for (uint32_t w = 1; w <= 4; w++) S.step_events.push_back(float(left[w]));
         }
         // walker descriptors of the decoupled kernel (see SigSchedule)
         for (uint32_t t = 0; t < S.steps.size(); t++)
