@@ -156,8 +156,20 @@ static int validate_program(const Program &P, uint64_t n_det, uint64_t n_obs, ui
                 if ((b[2 * i] & 0x7FFFFFFFu) >= P.n_slots || b[2 * i + 1] >= n_meas) return bad(at + ": record out of range");
             break;
         case L_NAPPLY: {
-            if (ly.nwords || ly.aux >= P.noise.size()) return bad(at + ": apply layer");
-            if (uint64_t(ly.aux2) + P.noise[ly.aux].n_seg > P.max_window_segs) return bad(at + ": window base");
+            if (!ly.count || 4ull * ly.count > ly.nwords) return bad(at + ": apply layer");
+            uint64_t seg = ly.aux2;
+            for (uint32_t i = 0; i < ly.count; i++) {
+                const uint32_t *r = b + 4 * i;
+                if (r[3] >= P.noise.size()) return bad(at + ": apply descriptor");
+                const NoiseDesc &nd = P.noise[r[3]];
+                const uint64_t words = uint64_t(nd.kind == N_DEP2 ? 2 : 1) * nd.n_units;
+                const bool in_block = (r[1] >> 31) != 0;
+                if (r[0] != seg || (r[1] & 0x7FFFFFFFu) != nd.kind) return bad(at + ": apply record");
+                if (in_block ? (uint64_t(r[2]) + words > ly.nwords || ly.off + r[2] != nd.tgt_off) : r[2] != nd.tgt_off)
+                    return bad(at + ": apply targets");
+                seg += nd.n_seg;
+            }
+            if (seg != uint64_t(ly.aux2) + ly.aux || seg > P.max_window_segs) return bad(at + ": window base");
             break;
         }
         default:
@@ -215,9 +227,12 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
     // and a record's frame word is not written again. Measurement program of
     // the d=11 non-local CNOT, 1e5 shots: 13.8 ms target by target, 0.99
     // grouped.
-    std::vector<uint32_t> op_gauges;
-    auto flush_gauges = [&](uint32_t op, uint32_t first = 0) {
-        for (uint32_t a = 0; a < op_gauges.size(); a++) gauge(op_gauges[a], op, first + a, ir);
+    struct PendingGauge {
+        uint32_t vreg, op, target;
+    };
+    std::vector<PendingGauge> op_gauges;
+    auto flush_gauges = [&]() {
+        for (const PendingGauge &g : op_gauges) gauge(g.vreg, g.op, g.target, ir);
         op_gauges.clear();
     };
     if (meas)
@@ -230,6 +245,9 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
     for (size_t i = 0; i < c->ops.size(); i++) {
         const HostOp &op = c->ops[i];
         const uint32_t *t = c->targets.data() + op.toff;
+        // resets in a row share their layers: their gauges wait for the next
+        // other op (a reset starts new frame words, so it never sees them)
+        if (op.code != TMCS_R && op.code != TMCS_RX) flush_gauges();
         switch (op.code) {
         case TMCS_R:
         case TMCS_RX:
@@ -238,10 +256,9 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
                 ir.push_back({I_ZERO, X[t[a]], 0});
                 Z[t[a]] = newv();
                 ir.push_back({I_ZERO, Z[t[a]], 0});
-                if (meas) op_gauges.push_back(op.code == TMCS_R ? Z[t[a]] : X[t[a]]);
-                if (!grouped) flush_gauges(uint32_t(i), a);
+                if (meas) op_gauges.push_back({op.code == TMCS_R ? Z[t[a]] : X[t[a]], uint32_t(i), a});
+                if (!grouped) flush_gauges();
             }
-            flush_gauges(uint32_t(i));
             break;
         case TMCS_H:
             for (uint32_t a = 0; a < op.nt; a++) std::swap(X[t[a]], Z[t[a]]);
@@ -264,13 +281,12 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
                 ir.push_back({I_COPY, nv, P[t[a]]});
                 P[t[a]] = nv;
                 if (meas && !grouped) ir.push_back({I_REC, rec[m], uint32_t(m)});
-                if (meas) op_gauges.push_back(op.code == TMCS_M ? Z[t[a]] : X[t[a]]);
-                if (!grouped) flush_gauges(uint32_t(i), a);
+                if (meas) op_gauges.push_back({op.code == TMCS_M ? Z[t[a]] : X[t[a]], uint32_t(i), a});
+                if (!grouped) flush_gauges();
                 m++;
             }
             if (meas && grouped)
                 for (uint32_t a = 0; a < op.nt; a++) ir.push_back({I_REC, rec[m - op.nt + a], uint32_t(m - op.nt + a)});
-            flush_gauges(uint32_t(i));
             break;
         case TMCS_X_ERROR:
         case TMCS_Z_ERROR:
@@ -642,13 +658,6 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
         const uint32_t nq = uint32_t(nz.comp.size() / 2);
         nd.n_units = nz.kind == N_DEP2 ? nq / 2 : nq;
         nd.n_seg = (nd.n_units + kSegUnits - 1) / kSegUnits;
-        nd.tgt_off = uint32_t(P.args.size());
-        for (uint32_t q = 0; q < nq; q++) {
-            uint32_t xs = nz.live[2 * q] ? slot[nz.comp[2 * q]] : kDeadSlot;
-            uint32_t zs = nz.live[2 * q + 1] ? slot[nz.comp[2 * q + 1]] : kDeadSlot;
-            P.args.push_back(xs | (zs << 16));
-            S.live_components += (xs != kDeadSlot) + (zs != kDeadSlot);
-        }
         noise_layer_desc[l] = uint32_t(P.noise.size());
         P.noise.push_back(nd);
         P.fault_base.push_back(op_fault_base[nz.op]);
@@ -679,6 +688,59 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
             i = j;
         }
     }
+    // Apply layers: noise ops that follow one another without an update in
+    // between (their events commute) and share a generation window are one
+    // layer. Its block holds a record per op and, where they fit, the ops'
+    // target words, so that applying an event reads shared memory only (a
+    // descriptor and then a target from L2, one after the other, made an
+    // apply layer about 1 us long whatever it did).
+    struct ApplyRun {
+        size_t off = 0;
+        uint32_t nwords = 0, count = 0, segs = 0;
+    };
+    std::vector<ApplyRun> apply_run(n_layers_body);
+    for (uint32_t l = 0; l < n_layers_body;) {
+        if (layer_kind[l] != I_NOISE) {
+            l++;
+            continue;
+        }
+        auto words_of = [&](uint32_t x) { return noise[ir[layer_insts[x][0]].a].comp.size() / 2; };
+        uint32_t e = l + 1;
+        size_t words = words_of(l);
+        while (e < n_layers_body && layer_kind[e] == I_NOISE &&
+               desc_win_first[noise_layer_desc[e]] == desc_win_first[noise_layer_desc[l]] &&
+               words + words_of(e) + 4 * (e - l + 1) + 4 <= kStageWords)
+            words += words_of(e++);
+        ApplyRun &R = apply_run[l];
+        R.count = e - l;
+        const bool in_block = words + 4 * R.count + 4 <= kStageWords;
+        pad4();
+        R.off = P.args.size();
+        P.args.resize(P.args.size() + 4 * R.count, 0u);
+        for (uint32_t x = l; x < e; x++) {
+            NoiseDesc &nd = P.noise[noise_layer_desc[x]];
+            const IRNoise &nz = noise[ir[layer_insts[x][0]].a];
+            nd.tgt_off = uint32_t(P.args.size());
+            for (size_t q = 0; 2 * q < nz.comp.size(); q++) {
+                const uint32_t xs = nz.live[2 * q] ? slot[nz.comp[2 * q]] : kDeadSlot;
+                const uint32_t zs = nz.live[2 * q + 1] ? slot[nz.comp[2 * q + 1]] : kDeadSlot;
+                P.args.push_back(xs | (zs << 16));
+                S.live_components += (xs != kDeadSlot) + (zs != kDeadSlot);
+            }
+            uint32_t *r = &P.args[R.off + 4 * (x - l)];
+            r[0] = desc_win_base[noise_layer_desc[x]];
+            r[1] = nd.kind | (in_block ? 0x80000000u : 0u);
+            r[2] = in_block ? nd.tgt_off - uint32_t(R.off) : nd.tgt_off;
+            r[3] = noise_layer_desc[x];
+            R.segs += nd.n_seg;
+            if (x == l && !in_block) R.nwords = 4 * R.count;
+        }
+        if (in_block) {
+            pad4();
+            R.nwords = uint32_t(P.args.size() - R.off);
+        }
+        l = e;
+    }
     for (uint32_t l = 0; l < n_layers_body; l++) {
         const std::vector<uint32_t> &ins = layer_insts[l];
         switch (layer_kind[l]) {
@@ -702,7 +764,12 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
         case I_NOISE: {
             const uint32_t d = noise_layer_desc[l];
             if (desc_win_first[d] == d) push_layer(L_NGEN, desc_win_count[d], 0, d, desc_win_segs[d], false);
-            push_layer(L_NAPPLY, 1, 0, d, desc_win_base[d], false);
+            const ApplyRun &R = apply_run[l];
+            if (R.count) {  // else: part of the run before
+                push_layer(L_NAPPLY, R.count, 0, R.segs, desc_win_base[d], false);
+                P.layers.back().off = uint32_t(R.off);
+                P.layers.back().nwords = R.nwords;
+            }
             break;
         }
         case I_GAUGE: {

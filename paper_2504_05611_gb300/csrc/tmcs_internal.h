@@ -29,8 +29,11 @@ enum LayerKind : uint32_t {
     L_COPY = 2,    // block[i] = dst | src << 16               -> dst = src
     L_NGEN = 3,    // walk the event streams of noise descriptors aux .. aux+count-1
                    // (a window of aux2 segments in total) into the event buffer
-    L_NAPPLY = 4,  // apply the buffered events of noise descriptor aux, whose
-                   // segments start at window segment aux2
+    L_NAPPLY = 4,  // apply the buffered events of count noise ops in a row: aux
+                   // window segments from aux2 on. block[4i..4i+3] = first
+                   // window segment of op i, kind | 0x80000000 if its targets
+                   // lie in the block, offset of its targets (in the block or
+                   // in args), descriptor
     L_DET = 5,     // block[0..count] = list bounds relative to the block; lists
                    // of record slots; detector ids aux .. aux+count-1
     L_OBS = 6,     // as L_DET; list[0] = accumulator slot, rest = record slots

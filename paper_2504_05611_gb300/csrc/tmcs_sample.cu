@@ -124,20 +124,25 @@ __device__ __forceinline__ void xor_bit(uint64_t *F, uint32_t slot, uint32_t K, 
 
 // One event of a noise op: Pauli index pk applied to the live frame
 // components of the unit's target(s) in lane pos % 64 of chunk word k.
-template <int K>
-__device__ __forceinline__ void apply_event(uint64_t *F, const uint32_t *__restrict__ tg, uint32_t kind,
-                                            uint32_t s, int pos, uint32_t pk, int k) {
+// SM: the targets lie in shared memory.
+template <int K, bool SM = false>
+__device__ __forceinline__ void apply_event(uint64_t *F, const uint32_t *tg, uint32_t kind, uint32_t s, int pos,
+                                            uint32_t pk, int k) {
+    auto ld = [](const uint32_t *a) -> uint32_t {
+        if constexpr (SM) return *a;
+        else return __ldg(a);
+    };
     const uint32_t unit = s * kSegUnits + uint32_t(pos >> 6);
     const unsigned long long bit = 1ull << (pos & 63);
     if (kind == N_DEP2) {
-        const uint32_t c0 = __ldg(tg + 2 * unit), c1 = __ldg(tg + 2 * unit + 1);
+        const uint32_t c0 = ld(tg + 2 * unit), c1 = ld(tg + 2 * unit + 1);
         const uint32_t pa = pk >> 2, pb = pk & 3u;
         if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, bit);
         if (pa & 2u) xor_bit(F, c0 >> 16, K, k, bit);
         if (pb & 1u) xor_bit(F, c1 & 0xFFFFu, K, k, bit);
         if (pb & 2u) xor_bit(F, c1 >> 16, K, k, bit);
     } else {
-        const uint32_t c0 = __ldg(tg + unit);
+        const uint32_t c0 = ld(tg + unit);
         const uint32_t pa = kind == N_XERR ? 1u : kind == N_ZERR ? 2u : pk;  // DEPOLARIZE1, PAULI_CHANNEL_1: pk
         if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, bit);
         if (pa & 2u) xor_bit(F, c0 >> 16, K, k, bit);
@@ -207,6 +212,44 @@ __device__ __forceinline__ void inject_faults(uint64_t *F, const KernelArgs &P, 
         const uint64_t idx = f - fb;
         const uint32_t unit = uint32_t(idx / KP), pk = uint32_t(idx % KP) + 1u;
         apply_event<K>(F, tg, nd.kind, unit / kSegUnits, int((unit % kSegUnits) * 64u + lane), pk, k);
+    }
+}
+
+// One apply layer (L_NAPPLY, its block at st): thread i of n takes event slots
+// i, i + n, ... of the layer's (segment, chunk) units; a walk that overflowed
+// its buffer resumes here. In single-fault mode the ops inject their faults.
+template <int K>
+__device__ __forceinline__ void apply_layer(uint64_t *F, const KernelArgs &P, const Layer &ly, const uint32_t *st,
+                                            EvUnit *evbuf, uint64_t col0, uint32_t chunk0, int nvalid, uint32_t i0,
+                                            uint32_t n) {
+    if (P.fault_mode) {
+        for (uint32_t r = 0; r < ly.count; r++) inject_faults<K>(F, P, st[4 * r + 3], col0, nvalid, i0, n);
+        return;
+    }
+    const uint32_t items = ly.aux * K * kEvCap;
+    for (uint32_t i = i0; i < items; i += n) {
+        const uint32_t uu = i / kEvCap, e = i % kEvCap;
+        const uint32_t ws = ly.aux2 + uu / K;
+        const int k = int(uu % K);
+        if (k >= nvalid) continue;
+        const EvUnit *E = evbuf + ws * K + uint32_t(k);
+        const bool go_on = e == 0 && E->cont_d != 0xFFFFu;
+        if (e >= E->n && !go_on) continue;
+        uint32_t r = 0;
+        while (r + 1 < ly.count && st[4 * (r + 1)] <= ws) r++;
+        const uint32_t s = ws - st[4 * r], kind = st[4 * r + 1] & 0x7FFFFFFFu, off = st[4 * r + 2];
+        if (e < E->n) {
+            const uint32_t v = E->ev[e];
+            if (st[4 * r + 1] >> 31) apply_event<K, true>(F, st + off, kind, s, int(v & 0xFFFu), v >> 12, k);
+            else apply_event<K>(F, P.args + off, kind, s, int(v & 0xFFFu), v >> 12, k);
+        }
+        if (go_on) {
+            const NoiseDesc nd = P.noise[st[4 * r + 3]];
+            const uint32_t *Tt = P.tables + size_t(nd.table) * kTableWords;
+            const float inv = __uint_as_float(__ldg(Tt + kGapLen));
+            walk_segment<K>(nd, Tt, inv, s, chunk0 + uint32_t(k), P.key0, P.key1, E->cont_d, E->cont_pos, nullptr, F,
+                            P.args + nd.tgt_off, k);
+        }
     }
 }
 
@@ -329,33 +372,9 @@ __device__ __forceinline__ void run_tile(const KernelArgs P, uint64_t *F, uint32
                 }
                 break;
             }
-            case L_NAPPLY: {
-                if (P.fault_mode) {
-                    inject_faults<K>(F, P, ly.aux, col0, nvalid, tid, T_);
-                    break;
-                }
-                const NoiseDesc nd = P.noise[ly.aux];
-                const uint32_t *tg = P.args + nd.tgt_off;
-                const uint32_t items = nd.n_seg * K * kEvCap;
-                for (uint32_t i = tid; i < items; i += T_) {
-                    const uint32_t uu = i / kEvCap, e = i % kEvCap;
-                    const uint32_t s = uu / K;
-                    const int k = int(uu % K);
-                    if (k >= nvalid) continue;
-                    const EvUnit *E = evbuf + (ly.aux2 + s) * K + uint32_t(k);
-                    if (e < E->n) {
-                        const uint32_t v = E->ev[e];
-                        apply_event<K>(F, tg, nd.kind, s, int(v & 0xFFFu), v >> 12, k);
-                    }
-                    if (e == 0 && E->cont_d != 0xFFFFu) {
-                        const uint32_t *Tt = P.tables + size_t(nd.table) * kTableWords;
-                        const float inv = __uint_as_float(__ldg(Tt + kGapLen));
-                        walk_segment<K>(nd, Tt, inv, s, chunk0 + uint32_t(k), P.key0, P.key1, E->cont_d,
-                                        E->cont_pos, nullptr, F, tg, k);
-                    }
-                }
+            case L_NAPPLY:
+                apply_layer<K>(F, P, ly, st, evbuf, col0, chunk0, nvalid, tid, T_);
                 break;
-            }
             case L_DET: {
                 for (uint32_t d = tid; d < ly.count; d += T_) {
                     const uint32_t lo = st[d], hi = st[d + 1];
@@ -1456,35 +1475,9 @@ __device__ __forceinline__ void consumer_group(const KernelArgs &P, uint64_t *Fw
             }
             break;
         }
-        case L_NAPPLY: {
-            // apply the buffered events of one op (one thread per event slot);
-            // a walk that overflowed its buffer resumes here
-            if (P.fault_mode) {
-                inject_faults<KW>(Fw, P, cur.aux, col0, nvalid, gtid, GT);
-                break;
-            }
-            const NoiseDesc nd = P.noise[cur.aux];
-            const uint32_t *tg = P.args + nd.tgt_off;
-            const uint32_t items = nd.n_seg * KW * kEvCap;
-            for (uint32_t i = gtid; i < items; i += GT) {
-                const uint32_t uu = i / kEvCap, e = i % kEvCap;
-                const uint32_t sg = uu / KW;
-                const int k = int(uu % KW);
-                if (k >= nvalid) continue;
-                const EvUnit *E = evbuf + (cur.aux2 + sg) * KW + uint32_t(k);
-                if (e < E->n) {
-                    const uint32_t v = E->ev[e];
-                    apply_event<KW>(Fw, tg, nd.kind, sg, int(v & 0xFFFu), v >> 12, k);
-                }
-                if (e == 0 && E->cont_d != 0xFFFFu) {
-                    const uint32_t *Tt = P.tables + size_t(nd.table) * kTableWords;
-                    const float inv = __uint_as_float(__ldg(Tt + kGapLen));
-                    walk_segment<KW>(nd, Tt, inv, sg, chunk0 + uint32_t(k), P.key0, P.key1, E->cont_d,
-                                     E->cont_pos, nullptr, Fw, tg, k);
-                }
-            }
+        case L_NAPPLY:
+            apply_layer<KW>(Fw, P, cur, st, evbuf, col0, chunk0, nvalid, gtid, GT);
             break;
-        }
         case L_DET:
             for (uint32_t d = gtid; d < cur.count; d += GT) {
                 const uint32_t lo = st[d], hi = st[d + 1];
