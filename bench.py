@@ -665,7 +665,7 @@ def _kernel_sha(kernel=None):
     import hashlib
     h = hashlib.sha256()
     if kernel and kernel.startswith("flow_kernel"):
-        files = ("tmcs_flow.cu", "tmcs_device.cuh", "tmcs_internal.h", "tmcs_signature.cpp")
+        files = ("tmcs_flow.cuh", "tmcs_flow.cu", "tmcs_device.cuh", "tmcs_internal.h", "tmcs_signature.cpp")
     else:
         files = ("tmcs_sample.cu", "tmcs_device.cuh", "tmcs_internal.h", "tmcs_host.cpp", "tmcs_signature.cpp")
     for f in files:

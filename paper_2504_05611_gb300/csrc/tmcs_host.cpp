@@ -713,6 +713,7 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
             words += words_of(e++);
         ApplyRun &R = apply_run[l];
         R.count = e - l;
+        P.apply_words += 4 * R.count + 6;
         const bool in_block = words + 4 * R.count + 4 <= kStageWords;
         pad4();
         R.off = P.args.size();

@@ -58,7 +58,7 @@ struct Layer {
 };
 
 constexpr uint32_t kStageWords = 2048;  // 8 KB per staging buffer (two buffers)
-constexpr uint32_t kEvCap = 8;          // events buffered per (segment, chunk)
+constexpr uint32_t kEvCap = 11;         // events buffered per (segment, chunk)
 constexpr uint32_t kWindowSegs = 192;   // noise segments per generation window
 constexpr uint32_t kWindowOps = 16;     // noise ops per generation window
 
@@ -95,6 +95,7 @@ struct Program {
     std::vector<double> table_p;
     uint32_t n_slots = 0;
     uint32_t max_window_segs = 0;  // event-buffer size in segments
+    size_t apply_words = 0;        // words of args that apply-layer records take (padding included)
     uint64_t n_faults = 0;         // single faults of the whole op list (see tmcs_fault_count)
     uint64_t n_det = 0, n_obs = 0;
 };

@@ -58,14 +58,16 @@ struct KernelArgs {
 };
 
 // Buffered events of one (segment, chunk) of a noise op: up to kEvCap events
-// as (position in segment: 12 bits | Pauli index << 12); if the walk had more,
-// it resumes at draw cont_d from position cont_pos when the op is applied.
+// as (position in segment: 12 bits | Pauli index << 12). If the walk had
+// more, n has kEvMore set and the walk resumes when the op is applied, at
+// draw kEvCap from the last buffered event's position (every draw before was
+// an event). Room for 11 instead of 8: at p = 1e-3 one 64-unit segment in 800
+// goes on, not one in 32, so an apply layer seldom waits for a walk
+// (measurement records of the d=11 circuit: 607 -> 554 us).
+constexpr uint32_t kEvMore = 0x8000u;
 struct EvUnit {
     uint16_t ev[kEvCap];
     uint16_t n;
-    uint16_t cont_d;  // 0xFFFF: walk complete
-    int16_t cont_pos;
-    uint16_t pad;
 };
 static_assert(sizeof(EvUnit) == 24, "EvUnit layout");
 
@@ -118,8 +120,12 @@ __device__ __forceinline__ void prefetch_l1(const void *p) {
     asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
 }
 
-__device__ __forceinline__ void xor_bit(uint64_t *F, uint32_t slot, uint32_t K, int k, unsigned long long bit) {
-    if (slot != kDeadSlot) atomicXor(reinterpret_cast<unsigned long long *>(&F[slot * K + k]), bit);
+// Flips bit `lane` of chunk word k of a slot: a 32-bit atomic on its half of
+// the word (measurement records of the d=11 circuit: 554 us with 64-bit
+// atomics, 492 with 32-bit ones).
+__device__ __forceinline__ void xor_bit(uint64_t *F, uint32_t slot, uint32_t K, int k, uint32_t lane) {
+    if (slot != kDeadSlot)
+        atomicXor(reinterpret_cast<unsigned int *>(&F[slot * K + k]) + (lane >> 5), 1u << (lane & 31u));
 }
 
 // One event of a noise op: Pauli index pk applied to the live frame
@@ -133,19 +139,19 @@ __device__ __forceinline__ void apply_event(uint64_t *F, const uint32_t *tg, uin
         else return __ldg(a);
     };
     const uint32_t unit = s * kSegUnits + uint32_t(pos >> 6);
-    const unsigned long long bit = 1ull << (pos & 63);
+    const uint32_t lane = uint32_t(pos) & 63u;
     if (kind == N_DEP2) {
         const uint32_t c0 = ld(tg + 2 * unit), c1 = ld(tg + 2 * unit + 1);
         const uint32_t pa = pk >> 2, pb = pk & 3u;
-        if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, bit);
-        if (pa & 2u) xor_bit(F, c0 >> 16, K, k, bit);
-        if (pb & 1u) xor_bit(F, c1 & 0xFFFFu, K, k, bit);
-        if (pb & 2u) xor_bit(F, c1 >> 16, K, k, bit);
+        if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, lane);
+        if (pa & 2u) xor_bit(F, c0 >> 16, K, k, lane);
+        if (pb & 1u) xor_bit(F, c1 & 0xFFFFu, K, k, lane);
+        if (pb & 2u) xor_bit(F, c1 >> 16, K, k, lane);
     } else {
         const uint32_t c0 = ld(tg + unit);
         const uint32_t pa = kind == N_XERR ? 1u : kind == N_ZERR ? 2u : pk;  // DEPOLARIZE1, PAULI_CHANNEL_1: pk
-        if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, bit);
-        if (pa & 2u) xor_bit(F, c0 >> 16, K, k, bit);
+        if (pa & 1u) xor_bit(F, c0 & 0xFFFFu, K, k, lane);
+        if (pa & 2u) xor_bit(F, c0 >> 16, K, k, lane);
     }
 }
 
@@ -157,7 +163,7 @@ __device__ __forceinline__ uint32_t pauli_index(const NoiseDesc &nd, uint32_t np
 
 // Walks draws d = d0, d0+1, ... of one (segment, chunk) stream from position
 // pos. With buf != nullptr, events are stored until kEvCap are held (then the
-// resume point is recorded); with buf == nullptr they are applied to F.
+// unit is marked kEvMore); with buf == nullptr they are applied to F.
 template <int K>
 __device__ __forceinline__ void walk_segment(const NoiseDesc &nd, const uint32_t *__restrict__ T, float inv,
                                              uint32_t s, uint32_t chunk, uint32_t key0, uint32_t key1,
@@ -171,15 +177,12 @@ __device__ __forceinline__ void walk_segment(const NoiseDesc &nd, const uint32_t
         if (d == d0 || (d & 1u) == 0) w = philox4x32_10(d >> 1, chunk, nd.op_index, s, key0, key1);
         const uint32_t wg = (d & 1u) ? w.z : w.x;
         const uint32_t wp = (d & 1u) ? w.w : w.y;
-        const int prev = pos;
         pos += 1 + gap_count_fast<false>(T, inv, wg);
         if (pos >= n_trials) break;
         const uint32_t pk = pauli_index(nd, npauli, wp);
         if (buf) {
             if (n == kEvCap) {
-                buf->cont_d = uint16_t(d);
-                buf->cont_pos = int16_t(prev);
-                buf->n = uint16_t(n);
+                buf->n = uint16_t(n | kEvMore);
                 return;
             }
             buf->ev[n++] = uint16_t(uint32_t(pos) | (pk << 12));
@@ -188,10 +191,7 @@ __device__ __forceinline__ void walk_segment(const NoiseDesc &nd, const uint32_t
             apply_event<K>(F, tg, nd.kind, s, pos, pk, k);
         }
     }
-    if (buf) {
-        buf->n = uint16_t(n);
-        buf->cont_d = 0xFFFFu;
-    }
+    if (buf) buf->n = uint16_t(n);
 }
 
 // Single-fault mode: every lane of the tile whose fault index falls in this
@@ -233,12 +233,13 @@ __device__ __forceinline__ void apply_layer(uint64_t *F, const KernelArgs &P, co
         const int k = int(uu % K);
         if (k >= nvalid) continue;
         const EvUnit *E = evbuf + ws * K + uint32_t(k);
-        const bool go_on = e == 0 && E->cont_d != 0xFFFFu;
-        if (e >= E->n && !go_on) continue;
+        const uint32_t n_ev = E->n & (kEvMore - 1u);
+        const bool go_on = e == 0 && (E->n & kEvMore) != 0;
+        if (e >= n_ev) continue;
         uint32_t r = 0;
         while (r + 1 < ly.count && st[4 * (r + 1)] <= ws) r++;
         const uint32_t s = ws - st[4 * r], kind = st[4 * r + 1] & 0x7FFFFFFFu, off = st[4 * r + 2];
-        if (e < E->n) {
+        {
             const uint32_t v = E->ev[e];
             if (st[4 * r + 1] >> 31) apply_event<K, true>(F, st + off, kind, s, int(v & 0xFFFu), v >> 12, k);
             else apply_event<K>(F, P.args + off, kind, s, int(v & 0xFFFu), v >> 12, k);
@@ -247,8 +248,8 @@ __device__ __forceinline__ void apply_layer(uint64_t *F, const KernelArgs &P, co
             const NoiseDesc nd = P.noise[st[4 * r + 3]];
             const uint32_t *Tt = P.tables + size_t(nd.table) * kTableWords;
             const float inv = __uint_as_float(__ldg(Tt + kGapLen));
-            walk_segment<K>(nd, Tt, inv, s, chunk0 + uint32_t(k), P.key0, P.key1, E->cont_d, E->cont_pos, nullptr, F,
-                            P.args + nd.tgt_off, k);
+            walk_segment<K>(nd, Tt, inv, s, chunk0 + uint32_t(k), P.key0, P.key1, kEvCap, int(E->ev[kEvCap - 1] & 0xFFFu),
+                            nullptr, F, P.args + nd.tgt_off, k);
         }
     }
 }
@@ -361,7 +362,6 @@ __device__ __forceinline__ void run_tile(const KernelArgs P, uint64_t *F, uint32
                     EvUnit *E = evbuf + u;
                     if (k >= nvalid) {
                         E->n = 0;
-                        E->cont_d = 0xFFFFu;
                         continue;
                     }
                     const NoiseDesc nd = P.noise[di];
@@ -1464,7 +1464,6 @@ __device__ __forceinline__ void consumer_group(const KernelArgs &P, uint64_t *Fw
                 EvUnit *E = evbuf + u;
                 if (k >= nvalid) {
                     E->n = 0;
-                    E->cont_d = 0xFFFFu;
                     continue;
                 }
                 const NoiseDesc nd = P.noise[di];
@@ -2170,10 +2169,11 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
     // warps, 1024 threads. Circuits whose events flip many outputs (BB codes:
     // weight-6 checks, several observables) want more applier warps than the
     // surface-code ones.
-    if (ds)
+    // (One chunk per tile only where nothing larger fits: it never won.)
+    for (int k_min = 2; ds && k_min >= 1 && cands.empty(); k_min--)
         for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
             if (c->sig.sched[sched].lag) continue;
-            for (int K = 2; K <= 16; K *= 2)
+            for (int K = k_min; K <= 16; K *= 2)
                 for (int app : {8, 12, 16, 20, 24}) {
                     const LaunchShape cs = make_shape_flow(c, n_cols, lim, sched, K, 1024, app);
                     if (cs.mode == 7) cands.push_back(cs);
@@ -2899,7 +2899,8 @@ static int batch_sample_shared(const tmcs_job *jobs, size_t n_jobs, void *stream
 
 constexpr size_t kNoAllocBytes = size_t(8) << 20;  // 8 MiB: status word + one compiled program
 constexpr size_t kNoAllocStatusBytes = 256;
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
+constexpr size_t kNoAllocRecords = size_t(64) << 10;  // room on top for apply-layer records, which the limit leaves out
+static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes + kNoAllocRecords];
 
 constexpr int kNoAllocMaxDevices = 64;
 static std::mutex g_noalloc_mu;
@@ -2940,7 +2941,7 @@ static int sample_noalloc(const tmcs_circuit *c, uint64_t first_chunk, uint64_t 
     const size_t b_noise = align256(P.noise.size() * sizeof(NoiseDesc));
     const size_t b_tables = align256(P.tables.size() * 4);
     const size_t need = kNoAllocStatusBytes + b_layers + b_args + b_noise + b_tables;
-    if (need > kNoAllocBytes)
+    if (need > kNoAllocBytes + std::min(P.apply_words * 4, kNoAllocRecords))
         return fail(TMCS_E_INVALID, "compiled program needs " + std::to_string(need) +
                                         " bytes; the allocation-free entry point holds at most " +
                                         std::to_string(kNoAllocBytes) + " (use tmcs_sample_range)");
