@@ -983,10 +983,14 @@ cudaError_t flow_go(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
     if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, s.threads, s.smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    // a CTA of more than 512 threads at this register budget leaves no room
+    // for a second one; smaller ones are asked for
+    int per_sm = 1;
+    if (s.threads <= 512) {
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, s.threads, s.smem);
+        if (e != cudaSuccess) return e;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+    }
     const uint64_t grid = std::max<uint64_t>(1, std::min<uint64_t>(a.n_tiles, uint64_t(sms) * uint64_t(per_sm)));
     kern<<<unsigned(grid), s.threads, s.smem, st>>>(a);
     return cudaGetLastError();

@@ -173,6 +173,15 @@ def tmcs_circuit_info(handle: int) -> Dict[str, int]:
     return dict(zip(("n_qubits", "n_meas", "n_det", "n_obs", "device_bytes"), (x.value for x in v)))
 
 
+def _sizes(handle: int) -> Tuple[int, int]:
+    """(n_det, n_obs) of a compiled circuit: tmcs_circuit_info without its
+    dictionary, for calls that ask once per job."""
+    v = (ctypes.c_uint64 * 5)()
+    a = ctypes.addressof(v)
+    _check(lib().tmcs_circuit_info(handle, a, a + 8, a + 16, a + 24, a + 32))
+    return v[2], v[3]
+
+
 def tmcs_circuit_stats(handle: int) -> Dict[str, int]:
     s = _Stats()
     _check(lib().tmcs_circuit_stats(ctypes.c_void_p(handle), ctypes.byref(s)))
@@ -305,10 +314,10 @@ def tmcs_sample(handle: int, shots: int, seed: int, det, obs, stream=None) -> No
 
 
 def tmcs_sample_range(handle: int, first_chunk: int, shots: int, seed: int, det, obs, stream=None) -> None:
-    info = tmcs_circuit_info(handle)
+    n_det, n_obs = _sizes(handle)
     cols = (shots + 63) // 64
-    _check_size(det, info["n_det"], cols, "detector")
-    _check_size(obs, info["n_obs"], cols, "observable")
+    _check_size(det, n_det, cols, "detector")
+    _check_size(obs, n_obs, cols, "observable")
     _check(lib().tmcs_sample_range(ctypes.c_void_p(handle), first_chunk, shots, seed & (2 ** 64 - 1),
                                    _dev_ptr(det), _dev_ptr(obs), _stream_ptr(stream)))
 
@@ -379,10 +388,10 @@ def tmcs_batch_sample(jobs: Sequence[Tuple[int, int, int, object, object]], stre
     """jobs: (handle, shots, seed, det, obs) tuples."""
     arr = (_Job * max(len(jobs), 1))()
     for i, (h, shots, seed, det, obs) in enumerate(jobs):
-        info = tmcs_circuit_info(h)
+        n_det, n_obs = _sizes(h)
         cols = (shots + 63) // 64
-        _check_size(det, info["n_det"], cols, "detector")
-        _check_size(obs, info["n_obs"], cols, "observable")
+        _check_size(det, n_det, cols, "detector")
+        _check_size(obs, n_obs, cols, "observable")
         arr[i] = _Job(h, shots, seed & (2 ** 64 - 1), _dev_ptr(det), _dev_ptr(obs))
     _check(lib().tmcs_batch_sample(ctypes.byref(arr), len(jobs), _stream_ptr(stream)))
 
