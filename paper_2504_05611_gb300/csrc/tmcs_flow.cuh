@@ -47,6 +47,7 @@
 #include <type_traits>
 
 #include "tmcs_device.cuh"
+#include "tmcs_flow_step.h"
 #include "tmcs_internal.h"
 
 namespace tmcs {
@@ -96,7 +97,7 @@ struct FlowCtl {
     uint32_t abort;                // a bounded wait expired
     uint32_t app_stop;             // appliers leave (written by applier thread 0 before a barrier)
     // of step Q, in slot Q mod kFlowSlots:
-    uint32_t done[kFlowSlots];     // walked batches | finished blocks of put-aside streams << 16
+    uint32_t done[kFlowSlots];     // walked batches | units << 16 (finished blocks of put-aside streams, closing unit)
     uint32_t cnt[kFlowSlots];      // arena entries reserved by its events
     uint32_t left[kFlowSlots];     // streams put aside
     uint32_t blk[kFlowSlots][kFlowBlocks / 4];  // entries written per block of 32 (a byte each)
@@ -227,6 +228,30 @@ __device__ __forceinline__ bool flow_warp_wait(FlowCtl &C, uint32_t *status, uin
     __syncwarp();
     return ok != 0;
 }
+
+// Accesses to a step's slot by a whole walker warp (lane 0 does the atomics).
+struct FlowStepWarp {
+    FlowCtl &C;
+    uint32_t slot, lane;
+    __device__ __forceinline__ uint32_t add_batch() {
+        uint32_t old = 0;
+        __syncwarp();
+        if (lane == 0) old = atom_add_acq_rel_shared(&C.done[slot], 1u);
+        return __shfl_sync(0xFFFFFFFFu, old, 0);
+    }
+    __device__ __forceinline__ void add_unit() {
+        __syncwarp();
+        if (lane == 0) red_release_add_shared(&C.done[slot], 0x10000u);
+    }
+    __device__ __forceinline__ uint32_t left() { return ld_acquire_shared(&C.left[slot]); }
+};
+// The same by one applier thread.
+struct FlowStepThread {
+    FlowCtl &C;
+    uint32_t slot;
+    __device__ __forceinline__ uint32_t done() { return ld_acquire_shared(&C.done[slot]); }
+    __device__ __forceinline__ uint32_t left() { return ld_shared_volatile(&C.left[slot]); }
+};
 
 // Walker warps.
 //
@@ -488,7 +513,7 @@ struct FlowWalker {
         return fm ? (lo >> 5) << 2 | fm : 0u;
     }
 
-    // Finishes n streams put aside in block `blk` and counts the block.
+    // Finishes n streams put aside in block `blk` (the caller counts the block).
     __device__ __forceinline__ void finish_block(uint32_t blk, uint32_t n) const {
         __syncwarp();  // the entries, acquired by one lane
         const bool have = lane < n;
@@ -498,8 +523,6 @@ struct FlowWalker {
         const uint32_t item = item0 + (e >> 17) * IPB + (sl >> LK);
         const Stream s = open(item, sl & uint32_t(K - 1), have);
         finish(s, uint32_t(W), int(e & 0xFFFu), have);
-        __syncwarp();
-        if (lane == 0) red_release_add_shared(&C.done[Q & (kFlowSlots - 1u)], 0x10000u);
     }
 
     __device__ void run(uint32_t nt, uint32_t nv_last) {
@@ -555,16 +578,20 @@ struct FlowWalker {
             }
             // the batch is walked (release: its events and entries are in the
             // arena or the ring)
-            __syncwarp();
-            uint32_t old = 0;
-            if (lane == 0) old = atom_add_acq_rel_shared(&C.done[Q & (kFlowSlots - 1u)], 1u);
-            old = __shfl_sync(0xFFFFFFFFu, old, 0);
-            if (full & 1u) finish_block(full >> 2, 32u);
-            if (full & 2u) finish_block((full >> 2) + 1u, 32u);
-            if ((old & 0xFFFFu) == nb - 1u) {
-                const uint32_t n = min(ld_acquire_shared(&C.left[Q & (kFlowSlots - 1u)]), lcap);
-                if (n & 31u) finish_block(n >> 5, n & 31u);
-            }
+            FlowStepWarp step{C, Q & (kFlowSlots - 1u), lane};
+            flow_batch_walked(
+                step, nb, lcap,
+                [&]() {
+                    if (full & 1u) {
+                        finish_block(full >> 2, 32u);
+                        step.add_unit();
+                    }
+                    if (full & 2u) {
+                        finish_block((full >> 2) + 1u, 32u);
+                        step.add_unit();
+                    }
+                },
+                [&](uint32_t blk, uint32_t n) { finish_block(blk, n); });
         }
     }
 };
@@ -696,13 +723,8 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
             // appliers whether they go on (one value read after the barrier,
             // so every applier thread leaves or none does)
             if (at == 0) {
-                // all batches walked and every block of put-aside streams
-                // finished (their number is final once the batches are)
-                auto complete = [&]() {
-                    const uint32_t d = ld_acquire_shared(&C.done[slot]);
-                    return (d & 0xFFFFu) == need &&
-                           (need == 0u || (d >> 16) == (min(ld_shared_volatile(&C.left[slot]), S.slcap[q]) + 31u) / 32u);
-                };
+                FlowStepThread step{C, slot};
+                auto complete = [&]() { return flow_step_complete(step, need, S.slcap[q]); };
                 uint32_t stop = ld_shared_volatile(&C.abort);
                 if (!stop && !complete()) {
                     const uint64_t t0 = globaltimer_ns();
