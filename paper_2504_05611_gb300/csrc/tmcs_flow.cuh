@@ -274,8 +274,9 @@ struct FlowStepThread {
 // 310 of its 830 warp-instructions per iteration on per-lane bookkeeping:
 // refill, gate, grouping lanes by step, completion.
 // FAST: gap tables in shared memory, one table read per gap count, no
-// PAULI_CHANNEL_1 noise (a program without ebit decoherence, p above 2.1e-5);
-// the other cases share the general kernel (tables through L1). Two kernels
+// PAULI_CHANNEL_1 noise (a program without ebit decoherence, every p above
+// 2.1e-5); the other cases share the general kernel (tables through L1),
+// which counts gaps with one read in batches whose tables all allow it. Two kernels
 // instead of run-time branches: the walkers' code is about the size of the
 // instruction caches, and every branch not taken sits between the ones that
 // are (stalls without an instruction were 1.6 of 12.7 cycles per issue).
@@ -466,10 +467,11 @@ struct FlowWalker {
         emit<NE>(ev, live);
     }
 
-    // Runs the lanes with `walk` to the end of their streams, a call at a time.
-    __device__ __forceinline__ void finish(const Stream &s, uint32_t call, int pos, bool walk) const {
+    // Runs the lanes with `walk` to the end of their streams, a call at a
+    // time. near: every lane's table allows the one-read count.
+    __device__ __forceinline__ void finish(const Stream &s, uint32_t call, int pos, bool walk, bool near) const {
         while (__any_sync(0xFFFFFFFFu, walk)) {
-            if (FAST || A.near) window<1, true>(s, call, pos, walk);
+            if (FAST || near) window<1, true>(s, call, pos, walk);
             else window<1, false>(s, call, pos, walk);
             call++;
             walk = walk && pos < s.n_trials;
@@ -478,8 +480,9 @@ struct FlowWalker {
 
     // Puts the lanes' unfinished streams (mask um, not 0) aside. Returns the
     // blocks of 32 that are complete with them (bits 0 and 1: the block
-    // whose number is in the bits above and the next one; 0: none). Entry: position | lane << 12 |
-    // first-window calls - 1 << 17 | batch within the step << 19.
+    // whose number is in the bits above and the next one; 0: none). Entry:
+    // position | lane << 12 | batch within the step << 17. Only batches that
+    // had a first window put streams aside, so all tables here are near.
     __device__ __forceinline__ uint32_t put_aside(const Stream &s, uint32_t um, uint32_t b, int pos) const {
         const uint32_t slot = Q & (kFlowSlots - 1u), n = uint32_t(__popc(um));
         uint32_t base = 0;
@@ -509,7 +512,7 @@ struct FlowWalker {
         }
         const uint32_t fm = __ballot_sync(0xFFFFFFFFu, full);
         // the region's tail is full: finish in place
-        if (base + n > lcap) finish(s, uint32_t(W), pos, mine && idx >= lcap);
+        if (base + n > lcap) finish(s, uint32_t(W), pos, mine && idx >= lcap, true);
         return fm ? (lo >> 5) << 2 | fm : 0u;
     }
 
@@ -517,12 +520,13 @@ struct FlowWalker {
     __device__ __forceinline__ void finish_block(uint32_t blk, uint32_t n) const {
         __syncwarp();  // the entries, acquired by one lane
         const bool have = lane < n;
-        const uint32_t a = upos + cap + 32u * blk + lane;
-        const uint32_t e = have ? S.arena[a >= A.arena ? a - A.arena : a] : 0u;
+        // lanes without an entry take the last one's (its table is a near one)
+        const uint32_t a = upos + cap + 32u * blk + min(lane, n - 1u);
+        const uint32_t e = S.arena[a >= A.arena ? a - A.arena : a];
         const uint32_t sl = (e >> 12) & 31u;
         const uint32_t item = item0 + (e >> 17) * IPB + (sl >> LK);
         const Stream s = open(item, sl & uint32_t(K - 1), have);
-        finish(s, uint32_t(W), int(e & 0xFFFu), have);
+        finish(s, uint32_t(W), int(e & 0xFFFu), have, true);
     }
 
     __device__ void run(uint32_t nt, uint32_t nv_last) {
@@ -563,7 +567,12 @@ struct FlowWalker {
             const uint32_t it = item0 + b * IPB + (lane >> LK);
             const Stream s = open(min(it, item_end - 1u), k, it < item_end && k < nv);
             int pos = -1;
-            const bool near = FAST || A.near;
+            // The one-read count is a choice per batch: a table of p below
+            // 2.1e-5 in one noise op must not take the first window from
+            // every other stream (as one choice per launch did: d=11
+            // decoherence workload with aged-ebit ops of p = 1.5e-5, 1e6 shots,
+            // 433 us against 290; without the small p 291 us).
+            const bool near = FAST || A.near || __all_sync(0xFFFFFFFFu, fabsf(s.inv) < kNearInv);
             if (near) window<W, true>(s, 0u, pos, true);
             const bool unfinished = pos < s.n_trials && s.n_trials > 0;
             const uint32_t um = __ballot_sync(0xFFFFFFFFu, unfinished);
@@ -572,8 +581,8 @@ struct FlowWalker {
                 // finish in place when most lanes go on, when there was no
                 // first window (a table needs the two-read count), and when
                 // the batch number does not fit an entry
-                if (!near) finish(s, 0u, pos, unfinished);
-                else if (__popc(um) > 24 || b >= (1u << 15)) finish(s, uint32_t(W), pos, unfinished);
+                if (!near) finish(s, 0u, pos, unfinished, false);
+                else if (__popc(um) > 24 || b >= (1u << 15)) finish(s, uint32_t(W), pos, unfinished, true);
                 else full = put_aside(s, um, b, pos);
             }
             // the batch is walked (release: its events and entries are in the
