@@ -164,56 +164,55 @@ cudaError_t flow_batch(const std::vector<FlowJob> &jobs, int sms, cudaStream_t s
     struct Entry {
         const FlowJob *j;
         FlowArgs a;
+        uint8_t variant;
         double tile;  // relative time of a tile
     };
-    // one launch per kernel variant (and per kFlowBatchJobs jobs)
-    for (int variant = 0; variant < 4; variant++) {
-        const bool wide = (variant & 1) != 0, fast = (variant & 2) != 0;
-        std::vector<Entry> v;
-        int window = 1;
-        for (const FlowJob &j : jobs) {
-            const SigProgram &G = j.c->sig;
-            Entry e{&j, flow_args(G, uint32_t(j.c->n_obs), j.ds, j.shape, j.call), 0.0};
-            if (G.wide != wide || (e.a.smem_tables && e.a.near && !e.a.pc1) != fast) continue;
-            flow_columns(e.a, j.shape, j.call, 0, j.call.n_cols);
-            // batches, events and detectors of a tile, in walker-instruction
-            // terms, and the steps' hand-overs
-            const SigSchedule &S = G.sched[j.shape.sched];
-            double events = 0;
-            for (size_t k = 0; k < S.step_events.size(); k += 5) events += double(S.step_events[k]);
-            e.tile = 600.0 * double(batches_per_tile(S, kFlowBatchK)) +
-                     kFlowBatchK * (2.0 * events + 1.0 * double(G.n_det)) + 2000.0 * double(S.steps.size());
-            window = std::max(window, int(G.window_calls));
-            v.push_back(e);
+    std::vector<Entry> v;
+    v.reserve(jobs.size());
+    for (const FlowJob &j : jobs) {
+        const SigProgram &G = j.c->sig;
+        Entry e{&j, flow_args(G, uint32_t(j.c->n_obs), j.ds, j.shape, j.call), 0, 0.0};
+        const bool fast = e.a.smem_tables && e.a.near && !e.a.pc1;
+        e.variant = flow_batch_variant(G.wide, fast, int(G.window_calls));
+        flow_columns(e.a, j.shape, j.call, 0, j.call.n_cols);
+        // batches, events and detectors of a tile, in walker-instruction
+        // terms, and the steps' hand-overs (rough weights: they only divide
+        // the CTAs among the jobs)
+        const SigSchedule &S = G.sched[j.shape.sched];
+        double events = 0;
+        for (size_t k = 0; k < S.step_events.size(); k += 5) events += double(S.step_events[k]);
+        e.tile = 600.0 * double(batches_per_tile(S, kFlowBatchK)) +
+                 kFlowBatchK * (2.0 * events + 1.0 * double(G.n_det)) + 2000.0 * double(S.steps.size());
+        v.push_back(e);
+    }
+    for (size_t base = 0; base < v.size(); base += kFlowBatchJobs) {
+        const size_t n = std::min<size_t>(kFlowBatchJobs, v.size() - base);
+        // CTAs: one each, then one more for the job that would finish
+        // last, until every SM has one
+        std::vector<uint32_t> ctas(n, 1);
+        auto time = [&](size_t i, uint32_t c) {
+            const Entry &e = v[base + i];
+            return double((e.a.n_tiles + c - 1) / c) * e.tile;
+        };
+        for (uint32_t used = uint32_t(n); used < uint32_t(sms); used++) {
+            size_t worst = 0;
+            for (size_t i = 1; i < n; i++)
+                if (time(i, ctas[i]) > time(worst, ctas[worst])) worst = i;
+            if (ctas[worst] >= v[base + worst].a.n_tiles) break;
+            ctas[worst]++;
         }
-        for (size_t base = 0; base < v.size(); base += kFlowBatchJobs) {
-            const size_t n = std::min<size_t>(kFlowBatchJobs, v.size() - base);
-            // CTAs: one each, then one more for the job that would finish
-            // last, until every SM has one
-            std::vector<uint32_t> ctas(n, 1);
-            auto time = [&](size_t i, uint32_t c) {
-                const Entry &e = v[base + i];
-                return double((e.a.n_tiles + c - 1) / c) * e.tile;
-            };
-            for (uint32_t used = uint32_t(n); used < uint32_t(sms); used++) {
-                size_t worst = 0;
-                for (size_t i = 1; i < n; i++)
-                    if (time(i, ctas[i]) > time(worst, ctas[worst])) worst = i;
-                if (ctas[worst] >= v[base + worst].a.n_tiles) break;
-                ctas[worst]++;
-            }
-            FlowBatchArgs b;
-            std::memset(static_cast<void *>(&b), 0, sizeof(b));
-            size_t smem = 0;
-            for (size_t i = 0; i < n; i++) {
-                b.jobs[i] = v[base + i].a;
-                b.cta_begin[i + 1] = b.cta_begin[i] + ctas[i];
-                smem = std::max(smem, v[base + i].j->shape.smem);
-            }
-            b.n_jobs = uint32_t(n);
-            const cudaError_t e = flow_batch_launch(b, wide, fast, window, v[base].j->shape.threads, smem, st);
-            if (e != cudaSuccess) return e;
+        FlowBatchArgs b;
+        std::memset(static_cast<void *>(&b), 0, sizeof(b));
+        size_t smem = 0;
+        for (size_t i = 0; i < n; i++) {
+            b.jobs[i] = v[base + i].a;
+            b.variant[i] = v[base + i].variant;
+            b.cta_begin[i + 1] = b.cta_begin[i] + ctas[i];
+            smem = std::max(smem, v[base + i].j->shape.smem);
         }
+        b.n_jobs = uint32_t(n);
+        const cudaError_t e = flow_batch_launch(b, v[base].j->shape.threads, smem, st);
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

@@ -968,42 +968,29 @@ __global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_kernel(const __
 // run side by side and none waits for a launch of its own. The job table is
 // a kernel parameter, so a graph can hold the launch. Tiles of four chunks:
 // the jobs are those that do not fill the GPU alone.
+//
+// A job's variant (slot layout, fast or general walker, first window) is a
+// branch per CTA, so jobs of all kinds share the launch. One launch per
+// variant let the longest step chain of each kind follow the others': four
+// small circuits of four kinds 43.5 us against 31.7, a batch of 16
+// distance-5 to 9 and BB18 circuits 100 us against 80.
 constexpr int kFlowBatchK = 4;
 constexpr uint32_t kFlowBatchJobs = 64;
 struct FlowBatchArgs {
     FlowArgs jobs[kFlowBatchJobs];
     uint32_t cta_begin[kFlowBatchJobs + 1];  // first CTA of each job; [n_jobs] = all
     uint32_t n_jobs;
+    uint8_t variant[kFlowBatchJobs];         // flow_batch_variant
 };
 static_assert(sizeof(FlowBatchArgs) <= 32000, "the job table exceeds the kernel parameter limit");
 
-template <bool WIDE, bool FAST, int W>
-__global__ void __launch_bounds__(TMCS_FLOW_MAX_THREADS, 1) flow_batch_kernel(const __grid_constant__ FlowBatchArgs B) {
-    extern __shared__ __align__(128) uint64_t smem[];
-    __shared__ FlowCtl C;
-    uint32_t lo = 0, hi = B.n_jobs - 1u;
-    while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1u) / 2u;
-        if (B.cta_begin[mid] <= blockIdx.x) lo = mid;
-        else hi = mid - 1u;
-    }
-    flow_cta<kFlowBatchK, WIDE, FAST, W>(B.jobs[lo], smem, C, blockIdx.x - B.cta_begin[lo],
-                                         B.cta_begin[lo + 1u] - B.cta_begin[lo]);
+// The general kernel has windows of three calls here, the fast one of two and
+// three.
+inline uint8_t flow_batch_variant(bool wide, bool fast, int window) {
+    return uint8_t((wide ? 1 : 0) + (!fast ? 0 : window <= 2 ? 2 : 4));
 }
 
-template <bool WIDE, bool FAST, int W>
-cudaError_t flow_batch_go(const FlowBatchArgs &b, int threads, size_t smem, cudaStream_t st) {
-    auto kern = flow_batch_kernel<WIDE, FAST, W>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, int(cudaSharedmemCarveoutMaxShared));
-    if (e != cudaSuccess) return e;
-    kern<<<b.cta_begin[b.n_jobs], threads, smem, st>>>(b);
-    return cudaGetLastError();
-}
-// Dispatch over its variants (tmcs_flow_batch.cu).
-cudaError_t flow_batch_launch(const FlowBatchArgs &b, bool wide, bool fast, int window, int threads, size_t smem,
-                              cudaStream_t st);
+cudaError_t flow_batch_launch(const FlowBatchArgs &b, int threads, size_t smem, cudaStream_t st);
 
 // Launch of one kernel variant: a persistent grid of the CTAs that are
 // resident at once, never more than there are tiles.

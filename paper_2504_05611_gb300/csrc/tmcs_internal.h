@@ -363,7 +363,7 @@ struct FlowJob {
     FlowCall call;
 };
 int flow_batch_tile();
-// Runs all jobs in as few launches as their kernel variants allow.
+// Runs all jobs in one launch per 64 of them.
 cudaError_t flow_batch(const std::vector<FlowJob> &jobs, int sms, cudaStream_t st);
 cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds, const FlowShape &s,
                         const FlowCall &call, int sms, cudaStream_t st);
