@@ -60,8 +60,41 @@ bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int applie
     if (aforce >= int(kFlowMinArena) && uint32_t(aforce) < s.arena) s.arena = uint32_t(aforce) & ~3u;
     if (s.arena < kFlowMinArena) return false;
     s.smem = fixed + (s.smem_tables ? tabs : 0) + size_t(s.arena) * 4;
+    // regions of the largest step that the arena holds, and the relative time
+    // of a tile (see flow_shape_untimed)
+    const double regions = double(s.arena) / double(uint64_t(flow_event_cap(S.max_events * float(K))) +
+                                                    flow_aside_cap(S.max_left[s.window] * float(K), s.arena));
+    s.holds_step = regions >= 1.0;
+    s.cost = double(S.steps.size()) +
+             S.sum_events * double(K) / 700.0 * (regions < 1.0 ? 2.5 : regions < 3.0 ? 1.25 : 1.0);
     *out = s;
     return true;
+}
+
+// The ring of least cost: a hand-over per step, and the tile's events, which
+// take longer when the arena holds less than three regions (walkers and
+// appliers then take turns) and much longer when it holds less than one (the
+// events beyond a region wait in the walkers until their step is applied).
+// Times of a tile, us, with the steps of a tile and the regions held, for
+// rings of 4096 / 2048 / 1024 detectors (d=29: 4096 / 2048), K = 4:
+//   d=11, p = 1e-3:  21 (1, 2.5) /  21 (2, 6.5) / 24 (4, 16)
+//   d=11, p = 3e-3:  92 (1, 0.9) /  46 (2, 2.3) / 37 (4, 5.8)
+//   d=11, p = 1e-2: 289 (1, 0.3) / 306 (2, 0.7) / 130 (4, 1.9)
+//   d=21, p = 1e-3:  94 (6, 1.8) /  86 (12, 6.7) / 110 (42, 15)
+//   d=29, p = 1e-3: 197 (17, 1.8) / 244 (58, 6.4)
+//   BB144 teleport, p = 3e-3: 121 (1, 0.5) / 89 (2, 1.8) / 70 (5, 4.2)
+// The weights fit these and the same circuits at K = 1, 2 and 8: 1.2 us a
+// step, 1.7 ns an event.
+bool flow_shape_untimed(const tmcs_circuit *c, int K, int threads, int appliers, size_t budget, FlowShape *out) {
+    bool found = false;
+    for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
+        FlowShape s;
+        if (!flow_shape(c, sched, K, threads, appliers, budget, &s)) continue;
+        if (found && s.cost >= out->cost) continue;
+        *out = s;
+        found = true;
+    }
+    return found;
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link

@@ -112,6 +112,8 @@ struct FlowShape {
     int window = 1;           // Philox calls of a stream's first window (1..4)
     uint32_t arena = 0;       // event arena entries
     bool smem_tables = false; // gap tables staged in shared memory
+    bool holds_step = false;  // the arena holds the region of every step
+    double cost = 0;          // relative time of a tile, to compare schedules at one K
     size_t smem = 0;          // dynamic shared memory
 };
 
@@ -213,6 +215,8 @@ struct SigSchedule {
     // streams that do not end in a first window of 1, 2, 3, 4 calls; the
     // decoupled kernel sizes the step's arena region by them.
     std::vector<float> step_events;
+    float max_events = 0, max_left[5] = {};  // the largest of each over the steps (max_left by window)
+    double sum_events = 0;                   // expected events per chunk that flip something, all steps
     // Walker descriptors of the decoupled kernel, 8 words per item (no
     // dependence on the seed): hi and lo of 0xCD9E8D57 x op index (Philox
     // round 1), segment, first compact event slot, kind | npauli << 3 |
@@ -354,6 +358,8 @@ void free_device_programs(tmcs_circuit *c);
 // Decoupled event-signature kernel (tmcs_flow.cu). flow_shape fills *out for
 // the given schedule, chunks per tile, CTA size and applier warps if that shape fits `budget` bytes of dynamic shared memory.
 bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out);
+// The same on the schedule for a launch that nothing has been timed for.
+bool flow_shape_untimed(const tmcs_circuit *c, int K, int threads, int appliers, size_t budget, FlowShape *out);
 #ifdef __CUDACC__
 // One circuit of a batched launch of the decoupled kernel.
 struct FlowJob {

@@ -1946,23 +1946,31 @@ static LaunchShape make_shape_sig(const tmcs_circuit *c, uint64_t n_cols, const 
 }
 
 // Decoupled event-signature kernel (mode 7): one CTA per SM, K chunks per
-// tile, `appliers` of its warps apply steps, the others walk. mode = 0 when
-// the shape does not fit.
+// tile, `appliers` of its warps apply steps, the others walk.
+static LaunchShape flow_launch_shape(const FlowShape &f, uint64_t n_cols, const DeviceLimits &lim) {
+    LaunchShape s;
+    s.mode = 7;
+    s.flow = f;
+    s.sched = f.sched;
+    s.K = f.K;
+    s.threads = f.threads;
+    s.warps = f.appliers;
+    s.sms = lim.sms;
+    s.smem = f.smem;
+    s.smem_tables = f.smem_tables;
+    s.qcap = f.arena;
+    s.tiles = std::min<uint64_t>((n_cols + uint64_t(f.K) - 1) / uint64_t(f.K), uint64_t(lim.sms));
+    return s;
+}
+
+// The same for the given schedule, chunks per tile, CTA size and applier
+// warps. mode = 0 when the shape does not fit.
 static LaunchShape make_shape_flow(const tmcs_circuit *c, uint64_t n_cols, const DeviceLimits &lim, int sched, int K,
                                    int threads, int appliers) {
     LaunchShape s;
     s.mode = 0;
-    if (!flow_shape(c, sched, K, threads, appliers, lim.smem_optin - 1024, &s.flow)) return s;
-    s.mode = 7;
-    s.sched = sched;
-    s.K = K;
-    s.threads = threads;
-    s.warps = appliers;
-    s.sms = lim.sms;
-    s.smem = s.flow.smem;
-    s.smem_tables = s.flow.smem_tables;
-    s.qcap = s.flow.arena;
-    s.tiles = std::min<uint64_t>((n_cols + K - 1) / K, uint64_t(lim.sms));
+    FlowShape f;
+    if (flow_shape(c, sched, K, threads, appliers, lim.smem_optin - 1024, &f)) s = flow_launch_shape(f, n_cols, lim);
     return s;
 }
 
@@ -2321,9 +2329,11 @@ static LaunchShape choose_shape_sig(const tmcs_circuit *c, uint64_t n_cols, cons
 // (best K / best time / time at the K chosen, us): d=29, 677 chunks 2 / 384
 // / 384; d=29, 150 chunks 1 / 126 / 126; d=11, 1563 chunks 4 / 74 / 74;
 // d=11, 157 chunks 2 / 44 / 45; BB144 teleport, 1563 chunks 4 / 141 / 156.
-// The largest ring that fits: fewer steps, so fewer hand-overs (d=29, 677
-// chunks, K = 4: ring 4096 402, 2048 485). Events of the eight-row layout
-// cost the appliers more, so they get more warps. mode = 0: no shape fits.
+// The ring is flow_shape_untimed's. A tile whose steps do not fit the arena
+// on any ring is not taken while a smaller one's do: at p = 1e-2 the product
+// rule alone took K = 8 for 1,216 chunks of d=11 (401 us, K = 2 254). Events
+// of the eight-row layout cost the appliers more, so they get more warps.
+// mode = 0: no shape fits.
 static LaunchShape choose_shape_flow(const tmcs_circuit *c, uint64_t n_cols, const DeviceLimits &lim) {
     LaunchShape best;
     best.mode = 0;
@@ -2332,14 +2342,11 @@ static LaunchShape choose_shape_flow(const tmcs_circuit *c, uint64_t n_cols, con
         const uint64_t tiles = (n_cols + uint64_t(K) - 1) / uint64_t(K);
         const uint64_t cost = (tiles + uint64_t(lim.sms) - 1) / uint64_t(lim.sms) * uint64_t(K + 1);
         if (best.mode && cost >= best_cost) continue;
-        for (int sched = 0; sched < int(c->sig.sched.size()); sched++) {
-            if (c->sig.sched[sched].lag) continue;
-            const LaunchShape s = make_shape_flow(c, n_cols, lim, sched, K, 1024, c->sig.wide ? 16 : 12);
-            if (s.mode != 7) continue;
-            best = s;
-            best_cost = cost;
-            break;
-        }
+        FlowShape f;
+        if (!flow_shape_untimed(c, K, 1024, c->sig.wide ? 16 : 12, lim.smem_optin - 1024, &f)) continue;
+        if (best.mode && !f.holds_step) break;  // nor do those of larger tiles
+        best = flow_launch_shape(f, n_cols, lim);
+        best_cost = cost;
     }
     return best;
 }
@@ -2578,8 +2585,8 @@ static cudaError_t launch_sig_batch(const SigBatchArgs &B, int threads, size_t s
     return cudaGetLastError();
 }
 
-// Batched launch through the decoupled kernel: every job on its largest ring
-// that fits, its CTAs side by side with the other jobs'. *used = false
+// Batched launch through the decoupled kernel: every job on the ring of an
+// untimed launch, its CTAs side by side with the other jobs'. *used = false
 // (nothing launched) if some job does not fit; the barrier kernel below then
 // takes the batch. 32 surface-code circuits of distance 3 to 9, 1e4 to 1e5
 // shots each: 207 us against 417 in the barrier kernel's shared launch.
@@ -2597,10 +2604,8 @@ static int flow_batch_sample(const tmcs_job *jobs, size_t n_jobs, cudaStream_t s
         if (!G.ok) return TMCS_OK;
         FlowJob f;
         f.c = J.c;
-        bool fits = false;
-        for (int sched = 0; sched < int(G.sched.size()) && !fits; sched++)
-            fits = !G.sched[sched].lag && flow_shape(J.c, sched, flow_batch_tile(), 1024, G.wide ? 16 : 12,
-                                                     lim.smem_optin - 1024, &f.shape);
+        const bool fits =
+            flow_shape_untimed(J.c, flow_batch_tile(), 1024, G.wide ? 16 : 12, lim.smem_optin - 1024, &f.shape);
         // batches and steps of a CTA are counted in 32 bits
         const uint64_t n_cols = (J.shots + 63) / 64;
         if (!fits || n_cols * (G.sched[f.shape.sched].items.size() / 2 + G.sched[f.shape.sched].steps.size()) >=

@@ -821,6 +821,9 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
             }
             S.step_events.push_back(float(ev));
             for (uint32_t w = 1; w <= 4; w++) S.step_events.push_back(float(left[w]));
+            S.max_events = std::max(S.max_events, float(ev));
+            S.sum_events += ev;
+            for (uint32_t w = 1; w <= 4; w++) S.max_left[w] = std::max(S.max_left[w], float(left[w]));
         }
         // walker descriptors of the decoupled kernel (see SigSchedule)
         for (uint32_t t = 0; t < S.steps.size(); t++)
