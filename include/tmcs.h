@@ -218,15 +218,16 @@ int tmcs_sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t shot
  * another allocator's pool, a real-time host that forbids allocation on its
  * request path, code that must not let cudaMalloc/cudaFree synchronise the
  * device -- it calls no cudaMalloc, cudaFree or other allocating routine.
- * Its scratch is one file-scope device array of 8 MiB (every GPU that loads
+ * Its scratch is one file-scope device array of 12.7 MiB (every GPU that loads
  * libtmcs.so holds it until the process exits): a status word (256 bytes)
  * followed by the circuit's compiled frame program, which each call copies
  * into it (stream-ordered on `stream`) before launching a frame kernel on it.
  * Every sampling kernel draws the same noise streams, so outputs are
  * bit-identical to tmcs_sample_range with the same arguments, whichever
  * kernel that call uses.
- *   - Circuits whose compiled program exceeds the array (device_bytes of
- *     tmcs_circuit_info plus 256) are rejected with TMCS_E_INVALID.
+ *   - Circuits whose compiled program exceeds 8 MiB (the status word and
+ *     device_bytes of tmcs_circuit_info, less its table of faults and what the
+ *     noise ops' application records take) are rejected with TMCS_E_INVALID.
  *   - The first call on each device looks up the array's device address with
  *     that device current and clears the status word (synchronously); make
  *     that first call before any stream capture.

@@ -699,6 +699,8 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
         uint32_t nwords = 0, count = 0, segs = 0;
     };
     std::vector<ApplyRun> apply_run(n_layers_body);
+    auto align4 = [](size_t n) { return (n + 3) & ~size_t(3); };
+    size_t plain_words = P.args.size();  // args with the targets alone
     for (uint32_t l = 0; l < n_layers_body;) {
         if (layer_kind[l] != I_NOISE) {
             l++;
@@ -713,7 +715,8 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
             words += words_of(e++);
         ApplyRun &R = apply_run[l];
         R.count = e - l;
-        P.apply_words += 4 * R.count + 6;
+        P.apply_merged += R.count - 1;
+        plain_words += words;
         const bool in_block = words + 4 * R.count + 4 <= kStageWords;
         pad4();
         R.off = P.args.size();
@@ -742,6 +745,7 @@ int compile(tmcs_circuit *c, uint32_t flags, bool meas, bool grouped) {
         }
         l = e;
     }
+    P.apply_words = align4(P.args.size()) - align4(plain_words);
     for (uint32_t l = 0; l < n_layers_body; l++) {
         const std::vector<uint32_t> &ins = layer_insts[l];
         switch (layer_kind[l]) {

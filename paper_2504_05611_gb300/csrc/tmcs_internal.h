@@ -95,7 +95,8 @@ struct Program {
     std::vector<double> table_p;
     uint32_t n_slots = 0;
     uint32_t max_window_segs = 0;  // event-buffer size in segments
-    size_t apply_words = 0;        // words of args that apply-layer records take (padding included)
+    size_t apply_words = 0;        // words of args that apply-layer records and their padding add
+    size_t apply_merged = 0;       // layers saved by applying noise ops in a row as one layer
     uint64_t n_faults = 0;         // single faults of the whole op list (see tmcs_fault_count)
     uint64_t n_det = 0, n_obs = 0;
 };

@@ -2910,7 +2910,10 @@ static int batch_sample_shared(const tmcs_job *jobs, size_t n_jobs, void *stream
 
 constexpr size_t kNoAllocBytes = size_t(8) << 20;  // 8 MiB: status word + one compiled program
 constexpr size_t kNoAllocStatusBytes = 256;
-constexpr size_t kNoAllocRecords = size_t(64) << 10;  // room on top for apply-layer records, which the limit leaves out
+// Room on top for the records of apply layers, which the limit leaves out: at
+// most ten words (four, and six of padding) for an op that takes a layer, a
+// descriptor and a target word of the limit, and one alignment of args.
+constexpr size_t kNoAllocRecords = kNoAllocBytes / (sizeof(Layer) + sizeof(NoiseDesc) + 4) * 40 + 512;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes + kNoAllocRecords];
 
 constexpr int kNoAllocMaxDevices = 64;
@@ -2952,8 +2955,11 @@ static int sample_noalloc(const tmcs_circuit *c, uint64_t first_chunk, uint64_t 
     const size_t b_noise = align256(P.noise.size() * sizeof(NoiseDesc));
     const size_t b_tables = align256(P.tables.size() * 4);
     const size_t need = kNoAllocStatusBytes + b_layers + b_args + b_noise + b_tables;
-    if (need > kNoAllocBytes + std::min(P.apply_words * 4, kNoAllocRecords))
-        return fail(TMCS_E_INVALID, "compiled program needs " + std::to_string(need) +
+    // the limit is on the program with a layer per noise op and no records
+    const size_t plain = kNoAllocStatusBytes + align256((P.layers.size() + P.apply_merged) * sizeof(Layer)) +
+                         align256((P.args.size() - P.apply_words) * 4) + b_noise + b_tables;
+    if (plain > kNoAllocBytes || need > sizeof(g_noalloc_scratch))
+        return fail(TMCS_E_INVALID, "compiled program needs " + std::to_string(plain) +
                                         " bytes; the allocation-free entry point holds at most " +
                                         std::to_string(kNoAllocBytes) + " (use tmcs_sample_range)");
     if (shots == 0) return fail(TMCS_E_INVALID, "shots must be positive");

@@ -324,8 +324,8 @@ def tmcs_sample_range(handle: int, first_chunk: int, shots: int, seed: int, det,
 
 def tmcs_sample_noalloc(handle: int, first_chunk: int, shots: int, seed: int, det, obs, stream=None) -> None:
     """Allocation-free sampling (see include/tmcs.h): same bits as
-    tmcs_sample_range; its scratch is a fixed 8 MiB device array shared by
-    all calls, so calls overlapping on the GPU race."""
+    tmcs_sample_range; its scratch is a fixed device array (programs of up to
+    8 MiB) shared by all calls, so calls overlapping on the GPU race."""
     info = tmcs_circuit_info(handle)
     cols = (shots + 63) // 64
     _check_size(det, info["n_det"], cols, "detector")
