@@ -1722,6 +1722,11 @@ static int device_program(const tmcs_circuit *c, const DeviceProgram **out) {
     return upload_program(c, c->prog, c->dev, out);
 }
 
+static bool sig_on_device(const tmcs_circuit *c, int dev) {
+    std::lock_guard<std::mutex> lock(c->mu);
+    return c->dev_sig.count(dev) != 0;
+}
+
 // Upload (once per device) the event-signature program.
 static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
     int dev = 0;
@@ -2414,8 +2419,18 @@ static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t sh
             if (f.mode == 7) s = f;
         }
     }
+    // Fault signatures by scatter need the event table on the device. Where it
+    // cannot be brought there (the stream is being captured, or no memory is
+    // left for it) the frame program, uploaded above, gives the same bits.
     if (fault_mode && c->sig.ok && kmode != 3 && kmode != 4 && c->sig.n_event_slots == P.n_faults) {
-        if ((rc = device_sig(c, &ds))) return rc;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaStreamIsCapturing(st, &cap);
+        if (cap == cudaStreamCaptureStatusNone || sig_on_device(c, dp->device)) {
+            rc = device_sig(c, &ds);
+            if (rc && rc != TMCS_E_OOM) return rc;
+        }
+    }
+    if (fault_mode && ds) {
         cudaError_t e = cudaSuccess;
         if (c->n_det) e = cudaMemsetAsync(det, 0, size_t(c->n_det) * n_cols * 8, st);
         if (e == cudaSuccess && c->n_obs) e = cudaMemsetAsync(obs, 0, size_t(c->n_obs) * n_cols * 8, st);
