@@ -479,8 +479,8 @@ int tmcs_debug_gap_table(double p, uint32_t *table);
  * method 0 as the decoupled kernel's walkers count (one table read guided by
  * a float estimate when |1/log2(1-p)| < 32768, else method 1), 1 the
  * two-read count with neighbour walks, 2 the log estimate with neighbour
- * loops (kernels 3 to 6 count as method 0 does where one read is allowed,
- * else by method 2). words and counts are device pointers to n uint32
+ * loops, 4 as kernels 3 to 6 count (their own form of the one read where it
+ * is allowed, else method 2). words and counts are device pointers to n uint32
  * and n int32. Blocks until done (on `stream`). Exported so tests can check
  * every route against the definition, words at the table's boundaries
  * included. Errors: TMCS_E_INVALID (NULL pointer, p outside (0, 1], bad

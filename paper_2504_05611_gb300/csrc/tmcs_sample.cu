@@ -1615,8 +1615,8 @@ static size_t kernel_smem_bytes(uint32_t n_slots, uint32_t max_window_segs, int 
 // Gap counts of words w by the device routines the kernels use (method 0:
 // the decoupled kernel's walkers, one table read when |inv_log2| <
 // kNearInv, else the two-read count; 1: the two-read count; 2: the log
-// estimate with neighbour loops, which kernels 3 to 6 use where the one
-// read is not allowed); table in global memory.
+// estimate with neighbour loops; 4: gap_count_fast, as kernels 3 to 6 count:
+// their own form of the one read, or method 2); table in global memory.
 __global__ void gap_counts_kernel(const uint32_t *__restrict__ T, float inv, float c32, const uint32_t *__restrict__ w,
                                   uint64_t n, int method, int32_t *__restrict__ out) {
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += uint64_t(gridDim.x) * blockDim.x) {
@@ -1624,6 +1624,7 @@ __global__ void gap_counts_kernel(const uint32_t *__restrict__ T, float inv, flo
         int g;
         if (method == 0 && fabsf(inv) < kNearInv) g = gap_count_magic<false>(T, 0xFFFFFFFFu, inv, c32, x);
         else if (method <= 1) g = gap_count_est<false>(T, inv, c32, x);
+        else if (method == 4) g = gap_count_fast<false>(T, inv, x);
         else g = gap_count(T, inv, x);
         out[i] = g;
     }
@@ -3073,7 +3074,7 @@ int tmcs_fault_signatures(const tmcs_circuit *c, uint64_t first_fault, uint64_t 
 
 int tmcs_debug_gap_counts(double p, const uint32_t *words, uint64_t n, int32_t *counts, int method, void *stream) {
     if (!words || !counts) return fail(TMCS_E_INVALID, "null words or counts");
-    if (method < 0 || method > 2) return fail(TMCS_E_INVALID, "method must be 0, 1 or 2");
+    if (method < 0 || method == 3 || method > 4) return fail(TMCS_E_INVALID, "method must be 0, 1, 2 or 4");
     std::vector<uint32_t> tables;
     std::vector<double> table_p;
     uint32_t id = 0;

@@ -261,8 +261,8 @@ def tmcs_debug_gap_table(p: float) -> np.ndarray:
 def tmcs_debug_gap_counts(p: float, words, method: int = 0, stream=None):
     """Gap counts of `words` (a CUDA uint32 tensor, or int32 viewed as such)
     for probability p by the device routine `method` (0 the decoupled
-    kernel's walkers, 1 the two-read count, 2 kernels 3-6); returns an int32
-    CUDA tensor."""
+    kernel's walkers, 1 the two-read count, 2 the log estimate with neighbour
+    loops, 4 kernels 3-6); returns an int32 CUDA tensor."""
     import torch
     if not (isinstance(words, torch.Tensor) and words.is_cuda and words.is_contiguous() and
             words.element_size() == 4):
