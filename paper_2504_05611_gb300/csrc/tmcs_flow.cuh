@@ -520,9 +520,10 @@ struct FlowWalker {
     __device__ __forceinline__ void finish_block(uint32_t blk, uint32_t n) const {
         __syncwarp();  // the entries, acquired by one lane
         const bool have = lane < n;
-        // lanes without an entry take the last one's (its table is a near one)
-        const uint32_t a = upos + cap + 32u * blk + min(lane, n - 1u);
-        const uint32_t e = S.arena[a >= A.arena ? a - A.arena : a];
+        // lanes without an entry take the step's first stream, in the general
+        // kernel the last entry's (its table is a near one)
+        const uint32_t a = upos + cap + 32u * blk + (FAST ? lane : min(lane, n - 1u));
+        const uint32_t e = !FAST || have ? S.arena[a >= A.arena ? a - A.arena : a] : 0u;
         const uint32_t sl = (e >> 12) & 31u;
         const uint32_t item = item0 + (e >> 17) * IPB + (sl >> LK);
         const Stream s = open(item, sl & uint32_t(K - 1), have);
