@@ -166,8 +166,6 @@ __device__ __forceinline__ int gap_count_est(const uint32_t *__restrict__ T, flo
 // So with m = rint(est) the count is m or m - 1, and one comparison with
 // T[m] decides (clamping m to [1, kGapLen] keeps the answer right at both
 // ends). Same result as gap_count_t for every w of such a table.
-constexpr float kNearInv = 32768.0f;
-
 // gap_count_near on the table whose word T[g - 1] sits at tab[base1 + g]
 // (base1 = the table's first word index minus one, modulo 2^32), so a
 // caller walking many draws of one table forms the base once.

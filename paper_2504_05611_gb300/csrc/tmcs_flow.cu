@@ -55,6 +55,8 @@ bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int applie
     // gap tables in shared memory when that still leaves an arena of 8192
     // entries, else read through L1
     s.smem_tables = arena_for(fixed + tabs) >= 8192u;
+    s.fast = s.smem_tables && G.near && !G.pc1;
+    if (!s.fast) s.window = s.window <= 1 ? 1 : 3;  // the general kernel's windows
     s.arena = arena_for(fixed + (s.smem_tables ? tabs : 0));
     const int aforce = env_int_flow("TMCS_FLOW_ARENA", 0);  // tuning/testing knob: arena entries
     if (aforce >= int(kFlowMinArena) && uint32_t(aforce) < s.arena) s.arena = uint32_t(aforce) & ~3u;
@@ -154,14 +156,8 @@ static FlowArgs flow_args(const SigProgram &G, uint32_t n_obs, const DeviceSig *
     a.n_obs = n_obs;
     a.arena = s.arena;
     a.test_cap = uint32_t(std::max(0, env_int_flow("TMCS_TEST_FLOW_CAP", 0)));
-    a.pc1 = 0u;
-    for (const NoiseDesc &nd : G.noise) a.pc1 |= nd.kind == N_PC1 ? 1u : 0u;
-    a.near = 1u;
-    for (size_t t = kGapLen; t < G.tables.size(); t += kTableWords) {
-        float inv;
-        std::memcpy(&inv, &G.tables[t], 4);
-        if (!(std::fabs(inv) < kNearInv)) a.near = 0u;
-    }
+    a.pc1 = G.pc1 ? 1u : 0u;
+    a.near = G.near ? 1u : 0u;
     a.smem_tables = s.smem_tables ? uint32_t(G.tables.size() / kTableWords) : 0u;
     a.walkers = uint32_t(s.threads / 32 - s.appliers);
     a.key0 = call.key0;
@@ -205,8 +201,7 @@ cudaError_t flow_batch(const std::vector<FlowJob> &jobs, int sms, cudaStream_t s
     for (const FlowJob &j : jobs) {
         const SigProgram &G = j.c->sig;
         Entry e{&j, flow_args(G, uint32_t(j.c->n_obs), j.ds, j.shape, j.call), 0, 0.0};
-        const bool fast = e.a.smem_tables && e.a.near && !e.a.pc1;
-        e.variant = flow_batch_variant(G.wide, fast, int(G.window_calls));
+        e.variant = flow_batch_variant(G.wide, j.shape.fast, j.shape.window);
         flow_columns(e.a, j.shape, j.call, 0, j.call.n_cols);
         // batches, events and detectors of a tile, in walker-instruction
         // terms, and the steps' hand-overs (rough weights: they only divide
@@ -281,14 +276,13 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     for (uint64_t c0 = 0; c0 < call.n_cols; c0 += slice_cols) {
         const uint64_t n = std::min(slice_cols, call.n_cols - c0);
         flow_columns(a, s, call, c0, n);
-        const bool fast = a.smem_tables && a.near && !a.pc1;
         cudaError_t e;
         switch (s.K) {
-        case 16: e = flow_go_16(a, s, G.wide, fast, sms, st); break;
-        case 8: e = flow_go_8(a, s, G.wide, fast, sms, st); break;
-        case 4: e = flow_go_4(a, s, G.wide, fast, sms, st); break;
-        case 2: e = flow_go_2(a, s, G.wide, fast, sms, st); break;
-        default: e = flow_go_1(a, s, G.wide, fast, sms, st); break;
+        case 16: e = flow_go_16(a, s, G.wide, sms, st); break;
+        case 8: e = flow_go_8(a, s, G.wide, sms, st); break;
+        case 4: e = flow_go_4(a, s, G.wide, sms, st); break;
+        case 2: e = flow_go_2(a, s, G.wide, sms, st); break;
+        default: e = flow_go_1(a, s, G.wide, sms, st); break;
         }
         if (e != cudaSuccess) return e;
     }

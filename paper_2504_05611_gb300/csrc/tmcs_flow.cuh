@@ -1026,8 +1026,8 @@ cudaError_t flow_go(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t
 // that they compile in parallel). The general kernel has windows of one and
 // three calls.
 template <int K, bool WIDE>
-cudaError_t flow_go_w(const FlowArgs &a, const FlowShape &s, bool fast, int sms, cudaStream_t st) {
-    if (!fast) return s.window <= 1 ? flow_go<K, WIDE, false, 1>(a, s, sms, st) : flow_go<K, WIDE, false, 3>(a, s, sms, st);
+cudaError_t flow_go_w(const FlowArgs &a, const FlowShape &s, int sms, cudaStream_t st) {
+    if (!s.fast) return s.window <= 1 ? flow_go<K, WIDE, false, 1>(a, s, sms, st) : flow_go<K, WIDE, false, 3>(a, s, sms, st);
     switch (s.window) {
     case 1: return flow_go<K, WIDE, true, 1>(a, s, sms, st);
     case 2: return flow_go<K, WIDE, true, 2>(a, s, sms, st);
@@ -1036,15 +1036,15 @@ cudaError_t flow_go_w(const FlowArgs &a, const FlowShape &s, bool fast, int sms,
     }
 }
 
-#define TMCS_FLOW_UNIT(K)                                                                                        \
-    cudaError_t flow_go_##K(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st) { \
-        return wide ? flow_go_w<K, true>(a, s, fast, sms, st) : flow_go_w<K, false>(a, s, fast, sms, st);         \
+#define TMCS_FLOW_UNIT(K)                                                                                  \
+    cudaError_t flow_go_##K(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st) {   \
+        return wide ? flow_go_w<K, true>(a, s, sms, st) : flow_go_w<K, false>(a, s, sms, st);               \
     }
 
-cudaError_t flow_go_1(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st);
-cudaError_t flow_go_2(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st);
-cudaError_t flow_go_4(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st);
-cudaError_t flow_go_8(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st);
-cudaError_t flow_go_16(const FlowArgs &a, const FlowShape &s, bool wide, bool fast, int sms, cudaStream_t st);
+cudaError_t flow_go_1(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st);
+cudaError_t flow_go_2(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st);
+cudaError_t flow_go_4(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st);
+cudaError_t flow_go_8(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st);
+cudaError_t flow_go_16(const FlowArgs &a, const FlowShape &s, bool wide, int sms, cudaStream_t st);
 
 }  // namespace tmcs

@@ -83,6 +83,9 @@ constexpr uint32_t kGapLen = 4096;     // T[1..4096]: a full segment has 4096 tr
 // word 4096 = float bits of 1/log2(1-p) (0 for p = 1), used only to guess the
 // count before the exact table check; words 4097..4099 = 0.
 constexpr uint32_t kTableWords = 4100;
+// Tables with |1/log2(1-p)| below this (p above about 2.1e-5) allow the
+// one-read gap count (derivation: tmcs_device.cuh).
+constexpr float kNearInv = 32768.0f;
 constexpr uint32_t kDeadSlot = 0xFFFFu;
 constexpr uint32_t kMaxSlots = 0xFFFEu;
 
@@ -110,7 +113,8 @@ struct FlowShape {
     int K = 4;                // chunks per tile
     int threads = 1024;
     int appliers = 8;         // applier warps (the other warps walk)
-    int window = 1;           // Philox calls of a stream's first window (1..4)
+    int window = 1;           // Philox calls of a stream's first window (1..4), as the kernel runs it
+    bool fast = false;        // the kernel without PAULI_CHANNEL_1, two-read counts and tables outside shared memory
     uint32_t arena = 0;       // event arena entries
     bool smem_tables = false; // gap tables staged in shared memory
     bool holds_step = false;  // the arena holds the region of every step
@@ -283,6 +287,8 @@ struct SigProgram {
     std::vector<uint32_t> compact_of;  // first CompactItem index of each descriptor's segments (0xFFFFFFFF: none)
     uint64_t n_compact_slots = 0;
     uint32_t window_calls = 1;         // Philox calls of a stream's first window in the decoupled kernel
+    bool pc1 = false;                  // has PAULI_CHANNEL_1 noise
+    bool near = true;                  // every gap table allows the one-read count
     bool wide = false;                 // eight rows per slot instead of four, up to 15 classes instead of 3
     double build_seconds = 0;
 };

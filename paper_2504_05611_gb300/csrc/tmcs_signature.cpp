@@ -199,10 +199,18 @@ static void build_compact(SigProgram &G, const std::vector<double> &table_p) {
         }
     }
     G.n_compact_slots = slots;
-    // (the general kernel -- PAULI_CHANNEL_1 noise, more gap tables than
-    // shared memory holds next to a ring -- has windows of 1 and 3 only)
-    bool general = G.tables.size() / kTableWords > 4;
-    for (const NoiseDesc &nd : G.noise) general = general || nd.kind == N_PC1;
+    G.pc1 = false;
+    for (const NoiseDesc &nd : G.noise) G.pc1 = G.pc1 || nd.kind == N_PC1;
+    G.near = true;
+    for (size_t t = kGapLen; t < G.tables.size(); t += kTableWords) {
+        float inv;
+        std::memcpy(&inv, &G.tables[t], 4);
+        G.near = G.near && std::fabs(inv) < kNearInv;
+    }
+    // (the general kernel -- PAULI_CHANNEL_1 noise, a p that needs the
+    // two-read count, more gap tables than shared memory holds next to a
+    // ring -- has windows of 1 and 3 only)
+    const bool general = G.tables.size() / kTableWords > 4 || G.pc1 || !G.near;
     G.window_calls = 1;
     for (uint32_t w = 2; w <= 4; w++)
         if ((!general || w == 3) && cost[w] < cost[G.window_calls]) G.window_calls = w;
