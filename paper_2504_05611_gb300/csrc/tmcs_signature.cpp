@@ -80,17 +80,15 @@ struct Pass {
 }  // namespace
 
 // Output list of event slot k (entries as in SigProgram::ev_ent).
-static void event_list(const SigProgram &G, size_t k, std::vector<uint32_t> &v) {
-    const uint32_t w0 = G.ev_ent[2 * k], w1 = G.ev_ent[2 * k + 1];
-    v.clear();
-    if (w0 == kEvNone) return;
-    if (w0 & kEvOverflow) {
-        const size_t off = w0 & ~kEvOverflow;
-        v.assign(G.ev_ent.begin() + off, G.ev_ent.begin() + off + w1);
-        return;
-    }
-    v.push_back(w0);
-    if (w1 != kEvNone) v.push_back(w1);
+struct EventList {
+    const uint32_t *at;
+    size_t n;
+};
+static EventList event_list(const SigProgram &G, size_t k) {
+    const uint32_t *w = &G.ev_ent[2 * k];
+    if (w[0] == kEvNone) return {w, 0};
+    if (w[0] & kEvOverflow) return {G.ev_ent.data() + (w[0] & ~kEvOverflow), w[1]};
+    return {w, w[1] == kEvNone ? size_t(1) : size_t(2)};
 }
 
 // Words of a compact event slot.
@@ -233,23 +231,22 @@ static bool build_rows(const SigProgram &G, uint64_t O, SigSchedule &S) {
     if (uint64_t(S.window) + O >= 0x7FFFu || G.n_compact_slots * wpr >= (uint64_t(1) << 30)) return false;
     const uint32_t spare = S.window + uint32_t(O), none = spare | (spare << 16);
     S.rows.assign(G.n_compact_slots * wpr, none);
-    std::vector<uint32_t> v;
     for (const CompactItem &it : G.compact) {
         const NoiseDesc &nd = G.noise[it.desc];
         const uint32_t KP = sig_paulis(nd.kind);
         const uint32_t u0 = it.seg * kSegUnits, units = std::min(kSegUnits, nd.n_units - u0);
         for (uint32_t u = 0; u < units; u++)
             for (uint32_t c = 1; c <= it.classes; c++) {
-                event_list(G, G.ev_base[it.desc] + size_t(u0 + u) * KP + (it.rep[c] - 1u), v);
+                const EventList v = event_list(G, G.ev_base[it.desc] + size_t(u0 + u) * KP + (it.rep[c] - 1u));
                 size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr;
-                for (uint32_t &e : v) e = row_of(e, S.window);
                 // chunks: all rows, or all but two and a link
-                for (size_t x = 0; x < v.size();) {
-                    const bool link = v.size() - x > 2 * wpr;
-                    const size_t n = link ? 2 * wpr - 2 : v.size() - x;
+                for (size_t x = 0; x < v.n;) {
+                    const bool link = v.n - x > 2 * wpr;
+                    const size_t n = link ? 2 * wpr - 2 : v.n - x;
                     for (size_t i = 0; i < n; i++, x++) {
+                        const uint32_t row = row_of(v.at[x], S.window);
                         uint32_t &w = S.rows[at + i / 2];
-                        w = (i & 1) ? (w & 0xFFFFu) | (v[x] << 16) : (w & 0xFFFF0000u) | v[x];
+                        w = (i & 1) ? (w & 0xFFFFu) | (row << 16) : (w & 0xFFFF0000u) | row;
                     }
                     if (!link) break;
                     const size_t chunk = S.rows.size() / wpr;
@@ -264,40 +261,66 @@ static bool build_rows(const SigProgram &G, uint64_t O, SigSchedule &S) {
     return true;
 }
 
-// Checks a barrier schedule's row table: every Pauli index of every unit
-// finds, through its segment's classes, exactly its own output list as rows
-// of the ring (an index of class 0 flips nothing).
-static std::string validate_rows(const SigProgram &G, uint64_t O, const SigSchedule &S) {
-    const size_t wpr = slot_words(G);
-    if (S.rows.size() < G.n_compact_slots * wpr || uint64_t(S.window) + O >= 0x7FFFu) return "row table size";
-    const uint32_t spare = S.window + uint32_t(O);
-    std::vector<uint32_t> v;
+// Checks the classes of every segment: every Pauli index of every unit has
+// the output list of its class's representative (an index of class 0 flips
+// nothing). With validate_rows, which checks the representatives' lists in
+// each schedule's row table, every index finds exactly its own list.
+static std::string validate_classes(const SigProgram &G) {
     for (const CompactItem &it : G.compact) {
         const NoiseDesc &nd = G.noise[it.desc];
         const uint32_t KP = sig_paulis(nd.kind);
         const uint32_t u0 = it.seg * kSegUnits, units = std::min(kSegUnits, nd.n_units - u0);
         if (it.slot0 + uint64_t(units) * it.classes > G.n_compact_slots) return "compact slot";
-        for (uint32_t u = 0; u < units; u++)
+        uint32_t cls[16] = {};
+        for (uint32_t k = 1; k <= KP; k++) {
+            cls[k] = uint32_t(it.lut >> (4 * (k - 1))) & 15u;
+            if (cls[k] > it.classes) return "event class";
+        }
+        for (uint32_t c = 1; c <= it.classes; c++)
+            if (it.rep[c] < 1 || it.rep[c] > KP || cls[it.rep[c]] != c) return "event class";
+        for (uint32_t u = 0; u < units; u++) {
+            const size_t e0 = G.ev_base[it.desc] + size_t(u0 + u) * KP - 1u;  // slot of index k: e0 + k
             for (uint32_t k = 1; k <= KP; k++) {
-                const size_t ek = G.ev_base[it.desc] + size_t(u0 + u) * KP + (k - 1u);
-                const uint32_t c = uint32_t(it.lut >> (4 * (k - 1))) & 15u;
-                if (c > it.classes) return "event class";
-                if (!c) {
-                    if (G.ev_ent[2 * ek] != kEvNone) return "event class";
+                const uint32_t *w = &G.ev_ent[2 * (e0 + k)];
+                if (!cls[k]) {
+                    if (w[0] != kEvNone) return "event class";
                     continue;
                 }
-                event_list(G, ek, v);
+                const uint32_t *r = &G.ev_ent[2 * (e0 + it.rep[cls[k]])];
+                if (w[0] == kEvNone && r[0] == kEvNone) continue;
+                if (w[0] == r[0] && w[1] == r[1]) continue;
+                const EventList a = event_list(G, e0 + k), b = event_list(G, e0 + it.rep[cls[k]]);
+                if (a.n != b.n || !std::equal(a.at, a.at + a.n, b.at)) return "event class";
+            }
+        }
+    }
+    return std::string();
+}
+
+// Checks a barrier schedule's row table: every class of every unit names the
+// rows of its representative's output list.
+static std::string validate_rows(const SigProgram &G, uint64_t O, const SigSchedule &S) {
+    const size_t wpr = slot_words(G);
+    if (S.rows.size() < G.n_compact_slots * wpr || uint64_t(S.window) + O >= 0x7FFFu) return "row table size";
+    const uint32_t spare = S.window + uint32_t(O);
+    for (const CompactItem &it : G.compact) {
+        const NoiseDesc &nd = G.noise[it.desc];
+        const uint32_t KP = sig_paulis(nd.kind);
+        const uint32_t u0 = it.seg * kSegUnits, units = std::min(kSegUnits, nd.n_units - u0);
+        for (uint32_t u = 0; u < units; u++)
+            for (uint32_t c = 1; c <= it.classes; c++) {
+                const EventList v = event_list(G, G.ev_base[it.desc] + size_t(u0 + u) * KP + (it.rep[c] - 1u));
                 size_t at = (it.slot0 + size_t(u) * it.classes + (c - 1u)) * wpr, x = 0;
                 for (;;) {
                     const uint32_t last = S.rows[at + wpr - 1];
                     const bool link = (last & kRowOverflow) != 0;
-                    if (link != (v.size() - x > 2 * wpr)) return "row list";
+                    if (link != (v.n - x > 2 * wpr)) return "row list";
                     const size_t n = link ? 2 * wpr - 2 : 2 * wpr;
                     for (size_t i = 0; i < n; i++) {
                         const uint32_t row = (S.rows[at + i / 2] >> (16 * (i & 1))) & 0xFFFFu;
                         // entries past the list name the spare row
-                        if (row != (x < v.size() ? row_of(v[x], S.window) : spare)) return "event row";
-                        if (x < v.size()) x++;
+                        if (row != (x < v.n ? row_of(v.at[x], S.window) : spare)) return "event row";
+                        if (x < v.n) x++;
                     }
                     if (!link) break;
                     at = size_t(last & ~kRowOverflow) * wpr;
@@ -371,6 +394,8 @@ static std::string validate_signature_program(const SigProgram &G, uint64_t D, u
             }
         }
     }
+    const std::string bad_classes = validate_classes(G);
+    if (!bad_classes.empty()) return bad_classes;
     for (const SigSchedule &S : G.sched) {
         const size_t n_items = S.items.size() / 2;
         const uint32_t W = S.window;
@@ -936,6 +961,22 @@ int build_signature_program(tmcs_circuit *c, uint32_t max_window) {
                     wd[k] &= wd[k] - 1u;
                     break;
                 }
+        } else if (what == "class") {
+            // a Pauli index, not the representative, in another class whose
+            // events flip other outputs
+            for (CompactItem &it : G.compact) {
+                uint32_t k = 1;
+                while (k <= 15 && ((it.lut >> (4 * (k - 1)) & 15u) != 1u || it.rep[1] == k)) k++;
+                if (it.classes < 2 || k > 15) continue;
+                const NoiseDesc &nd = G.noise[it.desc];
+                const size_t e0 = G.ev_base[it.desc] + size_t(it.seg) * kSegUnits * sig_paulis(nd.kind) - 1u;
+                const EventList a = event_list(G, e0 + it.rep[1]), b = event_list(G, e0 + it.rep[2]);
+                if (a.n == b.n && std::equal(a.at, a.at + a.n, b.at)) continue;
+                it.lut += uint64_t(1) << (4 * (k - 1));
+                break;
+            }
+        } else if (what == "row" && !G.sched.empty() && !G.sched[0].rows.empty()) {
+            G.sched[0].rows[0] ^= 1u;  // the first event's first output row
         }
     }
     const std::string bad = validate_signature_program(G, D, O);
