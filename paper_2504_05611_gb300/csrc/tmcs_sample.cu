@@ -1740,51 +1740,60 @@ static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
         return TMCS_OK;
     }
     const SigProgram &G = c->sig;
-    const size_t b_noise = align256(G.noise.size() * sizeof(NoiseDesc));
-    const size_t b_tables = align256(G.tables.size() * 4);
     const size_t n_sched = G.sched.size();
-    size_t b_items[kSigMaxSchedules] = {}, b_steps[kSigMaxSchedules] = {}, b_sev[kSigMaxSchedules] = {},
-           b_desc[kSigMaxSchedules] = {}, b_rows[kSigMaxSchedules] = {}, b_sched = 0;
-    for (size_t k = 0; k < n_sched; k++) {
-        b_items[k] = align256(G.sched[k].item_rec.size() * 4);
-        b_steps[k] = align256(G.sched[k].steps.size() * sizeof(SigStep));
-        b_sev[k] = align256(G.sched[k].step_events.size() * sizeof(float));
-        b_desc[k] = align256(G.sched[k].item_desc.size() * 4);
-        b_rows[k] = align256(G.sched[k].rows.size() * 4);
-        b_sched += b_items[k] + b_steps[k] + b_sev[k] + b_desc[k] + b_rows[k];
-    }
-    const size_t b_ent = align256(G.ev_ent.size() * 4);
-    const size_t total = std::max<size_t>(b_noise + b_tables + b_sched + b_ent, 256);
-    std::vector<uint8_t> host(total, 0);
-    size_t o = 0;
-    auto put = [&](const void *src, size_t n, size_t span) {
-        if (n) std::memcpy(host.data() + o, src, n);
-        const size_t at = o;
-        o += span;
-        return at;
-    };
     std::vector<NoiseDesc> dn = G.noise;
     for (size_t i = 0; i < dn.size(); i++) dn[i].tgt_off = G.ev_base[i];
-    const size_t o_noise = put(dn.data(), dn.size() * sizeof(NoiseDesc), b_noise);
-    const size_t o_tables = put(G.tables.data(), G.tables.size() * 4, b_tables);
-    size_t o_items[kSigMaxSchedules] = {}, o_steps[kSigMaxSchedules] = {}, o_sev[kSigMaxSchedules] = {},
-           o_desc[kSigMaxSchedules] = {}, o_rows[kSigMaxSchedules] = {};
-    for (size_t k = 0; k < n_sched; k++) {
-        const SigSchedule &S = G.sched[k];
-        o_items[k] = put(S.item_rec.data(), S.item_rec.size() * 4, b_items[k]);
-        o_steps[k] = put(S.steps.data(), S.steps.size() * sizeof(SigStep), b_steps[k]);
-        o_sev[k] = put(S.step_events.data(), S.step_events.size() * sizeof(float), b_sev[k]);
-        o_desc[k] = put(S.item_desc.data(), S.item_desc.size() * 4, b_desc[k]);
-        o_rows[k] = put(S.rows.data(), S.rows.size() * 4, b_rows[k]);
+    // One allocation. Small sections go through one host buffer and copy;
+    // large ones are copied from where they are (the event table and the rows
+    // of d=29 are 48 and 18 MB: filling a buffer with them first made a first
+    // call 9.2 ms, 1.9 now).
+    constexpr size_t kDirect = size_t(256) << 10;
+    struct Section {
+        const void *src;
+        size_t bytes, at;
+    };
+    std::vector<Section> secs;
+    auto put = [&](const void *src, size_t bytes) {
+        secs.push_back({src, bytes, 0});
+        return secs.size() - 1;
+    };
+    const size_t i_noise = put(dn.data(), dn.size() * sizeof(NoiseDesc));
+    const size_t i_tables = put(G.tables.data(), G.tables.size() * 4);
+    const size_t i_sched = secs.size();
+    for (const SigSchedule &S : G.sched) {
+        put(S.item_rec.data(), S.item_rec.size() * 4);
+        put(S.steps.data(), S.steps.size() * sizeof(SigStep));
+        put(S.step_events.data(), S.step_events.size() * sizeof(float));
+        put(S.item_desc.data(), S.item_desc.size() * 4);
+        put(S.rows.data(), S.rows.size() * 4);
     }
-    const size_t o_ent = put(G.ev_ent.data(), G.ev_ent.size() * 4, b_ent);
+    const size_t i_ent = put(G.ev_ent.data(), G.ev_ent.size() * 4);
+    size_t staged = 0;
+    for (Section &x : secs)
+        if (x.bytes < kDirect) {
+            x.at = staged;
+            staged += align256(x.bytes);
+        }
+    size_t total = staged;
+    for (Section &x : secs)
+        if (x.bytes >= kDirect) {
+            x.at = total;
+            total += align256(x.bytes);
+        }
+    total = std::max<size_t>(total, 256);
+    std::vector<uint8_t> host(staged, 0);
+    for (const Section &x : secs)
+        if (x.bytes && x.bytes < kDirect) std::memcpy(host.data() + x.at, x.src, x.bytes);
     void *base = nullptr;
     e = cudaMalloc(&base, total);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(TMCS_E_OOM, std::string("cudaMalloc of the signature program: ") + cudaGetErrorString(e));
     }
-    e = cudaMemcpy(base, host.data(), total, cudaMemcpyHostToDevice);
+    uint8_t *b = static_cast<uint8_t *>(base);
+    if (staged) e = cudaMemcpy(b, host.data(), staged, cudaMemcpyHostToDevice);
+    for (const Section &x : secs)
+        if (x.bytes >= kDirect && e == cudaSuccess) e = cudaMemcpy(b + x.at, x.src, x.bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(base);
         return cuda_fail(e, "cudaMemcpy of the signature program");
@@ -1793,17 +1802,17 @@ static int device_sig(const tmcs_circuit *c, const DeviceSig **out) {
     ds.device = dev;
     ds.base = base;
     ds.bytes = total;
-    uint8_t *b = static_cast<uint8_t *>(base);
-    ds.noise = reinterpret_cast<const NoiseDesc *>(b + o_noise);
-    ds.tables = reinterpret_cast<const uint32_t *>(b + o_tables);
+    ds.noise = reinterpret_cast<const NoiseDesc *>(b + secs[i_noise].at);
+    ds.tables = reinterpret_cast<const uint32_t *>(b + secs[i_tables].at);
     for (size_t k = 0; k < n_sched; k++) {
-        ds.items[k] = reinterpret_cast<const uint32_t *>(b + o_items[k]);
-        ds.steps[k] = reinterpret_cast<const SigStep *>(b + o_steps[k]);
-        ds.step_events[k] = reinterpret_cast<const float *>(b + o_sev[k]);
-        ds.item_desc[k] = reinterpret_cast<const uint32_t *>(b + o_desc[k]);
-        if (!G.sched[k].rows.empty()) ds.rows[k] = reinterpret_cast<const uint32_t *>(b + o_rows[k]);
+        const Section *x = &secs[i_sched + 5 * k];
+        ds.items[k] = reinterpret_cast<const uint32_t *>(b + x[0].at);
+        ds.steps[k] = reinterpret_cast<const SigStep *>(b + x[1].at);
+        ds.step_events[k] = reinterpret_cast<const float *>(b + x[2].at);
+        ds.item_desc[k] = reinterpret_cast<const uint32_t *>(b + x[3].at);
+        if (!G.sched[k].rows.empty()) ds.rows[k] = reinterpret_cast<const uint32_t *>(b + x[4].at);
     }
-    ds.ev_ent = reinterpret_cast<const uint32_t *>(b + o_ent);
+    ds.ev_ent = reinterpret_cast<const uint32_t *>(b + secs[i_ent].at);
     auto ins = c->dev_sig.emplace(dev, ds);
     *out = &ins.first->second;
     return TMCS_OK;
