@@ -62,13 +62,11 @@ bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int applie
     if (aforce >= int(kFlowMinArena) && uint32_t(aforce) < s.arena) s.arena = uint32_t(aforce) & ~3u;
     if (s.arena < kFlowMinArena) return false;
     s.smem = fixed + (s.smem_tables ? tabs : 0) + size_t(s.arena) * 4;
-    // regions of the largest step that the arena holds, and the relative time
-    // of a tile (see flow_shape_untimed)
-    const double regions = double(s.arena) / double(uint64_t(flow_event_cap(S.max_events * float(K))) +
-                                                    flow_aside_cap(S.max_left[s.window] * float(K), s.arena));
-    s.holds_step = regions >= 1.0;
+    s.regions = double(s.arena) / double(uint64_t(flow_event_cap(S.max_events * float(K))) +
+                                         flow_aside_cap(S.max_left[s.window] * float(K), s.arena));
+    // relative time of a tile (see flow_shape_untimed)
     s.cost = double(S.steps.size()) +
-             S.sum_events * double(K) / 700.0 * (regions < 1.0 ? 2.5 : regions < 3.0 ? 1.25 : 1.0);
+             S.sum_events * double(K) / 700.0 * (s.regions < 1.0 ? 2.5 : s.regions < 3.0 ? 1.25 : 1.0);
     *out = s;
     return true;
 }

@@ -117,7 +117,7 @@ struct FlowShape {
     bool fast = false;        // the kernel without PAULI_CHANNEL_1, two-read counts and tables outside shared memory
     uint32_t arena = 0;       // event arena entries
     bool smem_tables = false; // gap tables staged in shared memory
-    bool holds_step = false;  // the arena holds the region of every step
+    double regions = 0;       // regions of the largest step that the arena holds
     double cost = 0;          // relative time of a tile, to compare schedules at one K
     size_t smem = 0;          // dynamic shared memory
 };

@@ -2184,6 +2184,8 @@ uint32_t *device_status_word(int device) {
 // this call (the real launch overwrites them) and records the fastest per
 // chunk for the circuit on this device. Synchronous; runs once per circuit
 // and device.
+static bool flow_dense(const SigProgram &G);
+
 static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const DeviceLimits &lim, uint64_t n_cols,
                     cudaStream_t st, LaunchShape *best, const DeviceSig *ds) {
     const Program &P = c->prog;
@@ -2202,12 +2204,19 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
                     if (cs.mode == 7) cands.push_back(cs);
                 }
         }
-    // circuits it does not fit: every schedule of the signature program
-    // (barrier kernel for lag 0, pipelined kernel otherwise) x chunks per CTA
-    // x CTA size. Where both fit these lost on every measured workload (d=29
-    // 21.1 against 9.4 ms, BB144 teleport 6.9 against 2.6), so they are not
-    // timed there.
-    if (ds && cands.empty())
+    // circuits it does not fit, and dense ones whose steps the arena does not
+    // hold at four chunks: every schedule of the signature program (barrier
+    // kernel for lag 0, pipelined kernel otherwise) x chunks per CTA x CTA
+    // size. Elsewhere these lost on every measured workload (d=29 21.1
+    // against 9.4 ms, BB144 teleport 6.9 against 2.6; p up to 1e-2 for d=5 to
+    // 29 and BB144 by 1.2 to 3 times), so they are not timed there; dense
+    // ones gain from them (d=11, p = 0.05, 3e5 shots 3.3 ms against 2.9).
+    bool others = cands.empty();
+    if (ds && !others && flow_dense(c->sig)) {
+        others = true;
+        for (const LaunchShape &cs : cands) others = others && (cs.K < 4 || cs.flow.regions < 1.0);
+    }
+    if (ds && others)
         for (int sched = 0; sched < int(c->sig.sched.size()); sched++)
             for (int K = 1; K <= 16; K *= 2) {
                 if (!sig_fits(c, lim, K, sched)) break;
@@ -2239,17 +2248,18 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
         cudaEventDestroy(e0);
         return cuda_fail(e, "cudaEventCreate");
     }
+    const bool with_flow = !cands.empty() && cands[0].mode == 7;
     double best_per_chunk = 1e30;
     LaunchShape chosen = *best;
     for (const LaunchShape &full : cands) {
         const uint64_t per_tile = full.mode == 4 ? uint64_t(full.warps) * full.K : uint64_t(full.K);
-        // the decoupled kernel's shapes are all timed on the same columns: what
-        // a short run leaves dirty in L2 at its end is then the same for all
-        // of them (four tiles per SM of each shape's own size favoured small
+        // the decoupled kernel's shapes, and what they are compared with, are
+        // all timed on the same columns: what a short run leaves dirty in L2
+        // at its end is then the same for all of them (four tiles per SM of each shape's own size favoured small
         // tiles, which write less and leave a larger part of it unwritten:
         // d=29 at p=1e-4, 1e7 shots, K=4 33.5 ms against K=8 27.1 ms)
         const uint64_t cols =
-            std::min<uint64_t>(n_cols, uint64_t(4) * lim.sms * (full.mode == 7 ? uint64_t(16) : per_tile));
+            std::min<uint64_t>(n_cols, uint64_t(4) * lim.sms * (with_flow ? uint64_t(16) : per_tile));
         if (cols / per_tile < uint64_t(lim.sms)) continue;
         LaunchShape s = full;
         if (s.mode != 5 && s.mode != 7) s.tiles = (cols + per_tile - 1) / per_tile;
@@ -2346,24 +2356,59 @@ static LaunchShape choose_shape_sig(const tmcs_circuit *c, uint64_t n_cols, cons
 // d=11, 157 chunks 2 / 44 / 45; BB144 teleport, 1563 chunks 4 / 141 / 156.
 // The ring is flow_shape_untimed's. A tile whose steps do not fit the arena
 // on any ring is not taken while a smaller one's do: at p = 1e-2 the product
-// rule alone took K = 8 for 1,216 chunks of d=11 (401 us, K = 2 254). Events
-// of the eight-row layout cost the appliers more, so they get more warps.
-// mode = 0: no shape fits.
+// rule alone took K = 8 for 1,216 chunks of d=11 (401 us, K = 2 254); one
+// whose steps barely fit counts as slower (d=21, p = 0.03, 2,344 chunks:
+// K = 4, 1.0 regions, 9.9 ms; K = 2, 2.1 regions, 7.5). Events of the
+// eight-row layout cost the appliers more, so they get more warps. mode = 0:
+// no shape fits.
 static LaunchShape choose_shape_flow(const tmcs_circuit *c, uint64_t n_cols, const DeviceLimits &lim) {
     LaunchShape best;
     best.mode = 0;
-    uint64_t best_cost = 0;
+    double best_cost = 0;
     for (int K = 1; K <= 16; K *= 2) {
         const uint64_t tiles = (n_cols + uint64_t(K) - 1) / uint64_t(K);
-        const uint64_t cost = (tiles + uint64_t(lim.sms) - 1) / uint64_t(lim.sms) * uint64_t(K + 1);
+        const double cost = double((tiles + uint64_t(lim.sms) - 1) / uint64_t(lim.sms) * uint64_t(K + 1));
         if (best.mode && cost >= best_cost) continue;
         FlowShape f;
         if (!flow_shape_untimed(c, K, 1024, c->sig.wide ? 16 : 12, lim.smem_optin - 1024, &f)) continue;
-        if (best.mode && !f.holds_step) break;  // nor do those of larger tiles
+        if (best.mode && f.regions < 1.0) break;  // nor do those of larger tiles
+        const double full = f.regions < 1.3 ? 1.45 * cost : cost;
+        if (best.mode && full >= best_cost) continue;
         best = flow_launch_shape(f, n_cols, lim);
-        best_cost = cost;
+        best_cost = full;
     }
     return best;
+}
+
+// Programs of many events per stream (p above 0.02 or so): there the barrier
+// kernel can be the faster one when the arena holds fewer than two steps.
+// Not with eight rows per event slot: the barrier kernel's two-output slots
+// make it 1.2 to 5 times slower on BB codes at every p up to 0.2.
+static uint64_t sig_items(const SigProgram &G) { return std::max<uint64_t>(1, G.sched[0].items.size() / 2); }
+static bool flow_dense(const SigProgram &G) {
+    return !G.wide && G.sched[0].sum_events >= 80.0 * double(sig_items(G));
+}
+
+// Whether the barrier kernel's default shape takes less time than flow shape
+// f for an untimed call of a dense program. Estimates in ns per event of a
+// chunk, fitted to d=5 to 29 at p = 0.02 to 0.2 and 10 to 6,250 chunks:
+// decoupled kernel, per chunk in turn on an SM, 2.1 with a region in the
+// arena, 3.0 without (more for programs of few segments, which leave walkers
+// idle), 3.4 above 250 events a stream; barrier kernel 2.3 and 1.42 for each
+// chunk per SM (more for few segments). Measured, decoupled against barrier:
+// d=11, p = 0.1, 10 chunks 411 / 636 us, 1,250 chunks 3.8 / 2.1 ms; d=29,
+// p = 0.1, 1,250 chunks 65 / 33 ms.
+static bool barrier_is_faster(const tmcs_circuit *c, const FlowShape &f, uint64_t n_cols, const DeviceLimits &lim) {
+    const SigProgram &G = c->sig;
+    if (f.regions >= 2.0 || !flow_dense(G)) return false;
+    const double items = double(sig_items(G)), per_stream = G.sched[0].sum_events / items;
+    const double few = std::max(1.0, 456.0 / items);
+    const uint64_t tiles = (n_cols + uint64_t(f.K) - 1) / uint64_t(f.K);
+    const double turns = double((tiles + uint64_t(lim.sms) - 1) / uint64_t(lim.sms)) * f.K;
+    const double flow = turns * (f.regions < 1.0 ? std::max(3.0 * few, per_stream > 250 ? 3.4 : 0.0)
+                                                 : per_stream > 250 ? 3.4 : 2.1);
+    const double barrier = 2.3 + 1000.0 / items + 1.42 * few * double(n_cols) / double(lim.sms);
+    return barrier < flow;
 }
 
 static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t shots, uint64_t seed,
@@ -2417,7 +2462,7 @@ static int sample_range(const tmcs_circuit *c, uint64_t first_chunk, uint64_t sh
         DeviceProgram &mdp = c->dev[dp->device];
         if (mdp.tuned_mode == 0 && ds) {
             const LaunchShape f = choose_shape_flow(c, n_cols, lim);
-            if (f.mode == 7) s = f;
+            if (f.mode == 7 && !barrier_is_faster(c, f.flow, n_cols, lim)) s = f;
         }
         if (mdp.tuned_mode == 3) s = make_shape(P, n_cols, mdp.tuned_K, mdp.tuned_threads);
         if (mdp.tuned_mode == 4) s = make_shape_w(P, n_cols, mdp.tuned_K, mdp.tuned_warps, mdp.tuned_group);
@@ -2631,6 +2676,8 @@ static int flow_batch_sample(const tmcs_job *jobs, size_t n_jobs, cudaStream_t s
         f.c = J.c;
         const bool fits =
             flow_shape_untimed(J.c, flow_batch_tile(), 1024, G.wide ? 16 : 12, lim.smem_optin - 1024, &f.shape);
+        // dense programs whose steps the arena does not hold (see flow_dense)
+        if (fits && f.shape.regions < 1.0 && flow_dense(G)) return TMCS_OK;
         // batches and steps of a CTA are counted in 32 bits
         const uint64_t n_cols = (J.shots + 63) / 64;
         if (!fits || n_cols * (G.sched[f.shape.sched].items.size() / 2 + G.sched[f.shape.sched].steps.size()) >=
