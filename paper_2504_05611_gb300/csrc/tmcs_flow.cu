@@ -161,7 +161,7 @@ static FlowArgs flow_args(const SigProgram &G, uint32_t n_obs, const DeviceSig *
     a.key0 = call.key0;
     a.key1 = call.key1;
     a.keys = philox_keys(call.key0, call.key1);
-    a.ld = call.n_cols;
+    a.ld = call.ld ? call.ld : call.n_cols;
     a.status = call.status;
     return a;
 }
@@ -256,7 +256,7 @@ cudaError_t flow_launch(const SigProgram &G, uint32_t n_obs, const DeviceSig *ds
     const uint32_t al = s.K >= 16 ? 1u : 16u / uint32_t(std::max(s.K, 1));
     const uint32_t trows = (uint32_t(std::max(env_int_flow("TMCS_FLOW_TMA_ROWS", 64), 1)) + al - 1) / al * al;
     const int tma = env_int_flow("TMCS_FLOW_TMA", -1);
-    if ((tma > 0 || (tma < 0 && s.K >= 8)) && encode_det_map(&a.tmap, call.det, G.n_det, call.n_cols, s.K, trows))
+    if ((tma > 0 || (tma < 0 && s.K >= 8)) && encode_det_map(&a.tmap, call.det, G.n_det, a.ld, s.K, trows))
         a.tma_rows = trows;
     // A CTA counts its batches and its steps in 32 bits: a call with more
     // tiles per CTA than that allows runs as several launches over column

@@ -166,6 +166,7 @@ constexpr uint32_t kFlowMaxSteps = 1024;
 struct FlowCall {
     uint32_t key0 = 0, key1 = 0, first_chunk = 0;
     uint64_t n_cols = 0, last_mask = 0;
+    uint64_t ld = 0;  // words between output rows (0: n_cols)
     uint64_t *det = nullptr, *obs = nullptr;
     uint32_t *status = nullptr;
 };

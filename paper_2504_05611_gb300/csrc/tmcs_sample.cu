@@ -55,6 +55,7 @@ struct KernelArgs {
     const uint64_t *fault_base;
     uint64_t fault_first;
     uint32_t fault_mode;
+    uint64_t ld;           // decoupled kernel: words between output rows (0: n_cols)
 };
 
 // Buffered events of one (segment, chunk) of a noise op: up to kEvCap events
@@ -2088,6 +2089,7 @@ static cudaError_t launch(const KernelArgs &a0, const LaunchShape &s, cudaStream
         call.key1 = a0.key1;
         call.first_chunk = a0.first_chunk;
         call.n_cols = a0.n_cols;
+        call.ld = a0.ld;
         call.last_mask = a0.last_mask;
         call.det = a0.det;
         call.obs = a0.obs;
@@ -2265,6 +2267,7 @@ static int autotune(const tmcs_circuit *c, int device, KernelArgs a, const Devic
         if (s.mode != 5 && s.mode != 7) s.tiles = (cols + per_tile - 1) / per_tile;
         KernelArgs t = a;
         t.n_cols = cols;
+        t.ld = full.mode == 7 ? n_cols : 0;  // the call's row stride
         t.last_mask = ~uint64_t(0);
         float ms = 0.f;
         for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {
