@@ -23,6 +23,15 @@ static size_t flow_fixed_bytes(const SigProgram &G, int sched, uint32_t n_obs, i
     return flow_ring_bytes(S.window, n_obs, K) + flow_step_bytes(uint32_t(S.steps.size()));
 }
 
+// Arena region of a step with mu expected events and ml expected put-aside
+// streams (the kernel's formulas, flow_cta; in one function for both, the
+// kernel's set-up compiled to code that made it 0.6 % slower).
+static double flow_region(float mu, float ml, uint32_t arena) {
+    const double blocks = double((uint64_t(std::ceil(ml + 6.0f * std::sqrt(ml))) + 63u) & ~uint64_t(31));
+    return std::ceil(mu + 6.0 * std::sqrt(mu) + 64.0) +
+           std::min({blocks, double((arena / 4u) & ~31u), double(32u * kFlowBlocks)});
+}
+
 bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int appliers, size_t budget, FlowShape *out) {
     const SigProgram &G = c->sig;
     if (!G.ok || sched < 0 || size_t(sched) >= G.sched.size()) return false;
@@ -62,8 +71,7 @@ bool flow_shape(const tmcs_circuit *c, int sched, int K, int threads, int applie
     if (aforce >= int(kFlowMinArena) && uint32_t(aforce) < s.arena) s.arena = uint32_t(aforce) & ~3u;
     if (s.arena < kFlowMinArena) return false;
     s.smem = fixed + (s.smem_tables ? tabs : 0) + size_t(s.arena) * 4;
-    s.regions = double(s.arena) / double(uint64_t(flow_event_cap(S.max_events * float(K))) +
-                                         flow_aside_cap(S.max_left[s.window] * float(K), s.arena));
+    s.regions = double(s.arena) / flow_region(S.max_events * float(K), S.max_left[s.window] * float(K), s.arena);
     // relative time of a tile (see flow_shape_untimed)
     s.cost = double(S.steps.size()) +
              S.sum_events * double(K) / 700.0 * (s.regions < 1.0 ? 2.5 : s.regions < 3.0 ? 1.25 : 1.0);

@@ -875,16 +875,6 @@ __device__ __forceinline__ void flow_apply(const FlowArgs &A, const FlowSmem &S,
     if (tma && at < 32u) tma_wait_all();  // the tensor stores have written the outputs
 }
 
-// Capacity of a step's arena region: for mu expected events, mean + 6 sigma +
-// 64 (Poisson-like counts); for ml expected put-aside streams, whole blocks, at most
-// a quarter of the arena and the counted blocks.
-__host__ __device__ inline uint32_t flow_event_cap(float mu) { return uint32_t(ceilf(mu + 6.0f * sqrtf(mu) + 64.0f)); }
-__host__ __device__ inline uint32_t flow_aside_cap(float ml, uint32_t arena) {
-    uint32_t n = (uint32_t(ceilf(ml + 6.0f * sqrtf(ml))) + 63u) & ~31u;
-    if (n > ((arena / 4u) & ~31u)) n = (arena / 4u) & ~31u;
-    return n < 32u * kFlowBlocks ? n : 32u * kFlowBlocks;
-}
-
 // CTA size the kernel is compiled for (its register budget follows from it)
 #ifndef TMCS_FLOW_MAX_THREADS
 #define TMCS_FLOW_MAX_THREADS 1024
@@ -899,13 +889,16 @@ __device__ __forceinline__ void flow_cta(const FlowArgs &A, uint64_t *smem, Flow
     const uint32_t rows = A.window_mask + 1u;
     for (uint32_t i = tid; i < (rows + A.n_obs) * uint32_t(K); i += T_) S.ring[i] = 0ull;
     for (uint32_t i = tid; i < A.smem_tables * kTableWords; i += T_) S.stab[i] = __ldg(A.tables + i);
-    // batches per step (prefix sum below) and region capacities over K
-    // chunks, at most the arena; steps without items hold none
+    // batches per step (prefix sum below) and region capacities: mean + 6 sigma + 64 of the step's events over K
+    // chunks (Poisson-like counts), at most the arena; steps without items
+    // hold none (flow_region, tmcs_flow.cu, has the same formulas)
     for (uint32_t i = tid; i < A.n_steps; i += T_) {
         const uint4 st = __ldg(A.steps + i);
         const float mu = __ldg(A.step_events + 5 * i) * float(K), ml = __ldg(A.step_events + 5 * i + W) * float(K);
-        uint32_t cap = A.test_cap ? A.test_cap : flow_event_cap(mu);
-        const uint32_t lcap = st.y > st.x ? flow_aside_cap(ml, A.arena) : 0u;
+        uint32_t cap = A.test_cap ? A.test_cap : uint32_t(ceilf(mu + 6.0f * sqrtf(mu) + 64.0f));
+        // put-aside streams: whole blocks, at most a quarter of the arena
+        uint32_t lcap = min((uint32_t(ceilf(ml + 6.0f * sqrtf(ml))) + 63u) & ~31u, (A.arena / 4u) & ~31u);
+        lcap = st.y > st.x ? min(lcap, 32u * kFlowBlocks) : 0u;
         cap = st.y > st.x ? min(cap, A.arena - lcap) : 0u;
         S.bend[i] = (st.y - st.x + 32u / uint32_t(K) - 1u) / (32u / uint32_t(K));
         S.scap[i] = cap;
