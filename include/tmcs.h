@@ -176,9 +176,9 @@ int tmcs_reference_sample(const tmcs_circuit *c, uint8_t *meas_bits);
  * shared-memory arena, applier warps apply whole steps), TMCS_TILE_K,
  * TMCS_THREADS, TMCS_SIG_SCHED (signature schedule index), TMCS_FLOW_APPLIERS
  * and TMCS_FLOW_ARENA (kernel 7: applier warps, arena entries),
- * TMCS_FLOW_WINDOW (kernel 7: Philox calls per walker pass, 2 to 4),
- * TMCS_FLOW_GLOBAL_ARENA=1 and TMCS_FLOW_GARENA (kernel 7: the arena in a
- * per-stream global scratch buffer, its entries per CTA), TMCS_FLOW_TMA
+ * TMCS_FLOW_WINDOW (kernel 7: Philox calls of a stream's first window, 1 to
+ * 4; with PAULI_CHANNEL_1 noise, a p below 2.1e-5 or gap tables outside
+ * shared memory 1, or 3 for the others; a batched launch 2 or 3), TMCS_FLOW_TMA
  * and TMCS_FLOW_TMA_ROWS (kernel 7 with 8 or more chunks per tile, or any
  * even number with TMCS_FLOW_TMA=1, writes finished detector rows as 2D
  * tensor stores, boxes of that many rows (default 64) by the tile's chunks,
@@ -253,9 +253,11 @@ int tmcs_sample_noalloc(const tmcs_circuit *c, uint64_t first_chunk, uint64_t sh
  * X_ERROR/Z_ERROR, 3 for DEPOLARIZE1/PAULI_CHANNEL_1 with 1=X, 2=Z, 3=Y, 15
  * for DEPOLARIZE2 with k>>2 on the first and k&3 on the second target).
  * tmcs_fault_count gives the number of faults.
- * tmcs_fault_signatures propagates faults first_fault .. first_fault+n_faults-1
- * through the noiseless circuit, one fault per lane, with the sampling
- * kernels: lane l of word c of detector j (layout of tmcs_sample with
+ * tmcs_fault_signatures writes what faults first_fault .. first_fault+n_faults-1
+ * flip in the noiseless circuit, one fault per lane: scattered from the event
+ * table of the signature program, or (without one, or while the stream is
+ * captured and the table is not on the device) by the frame kernels, which
+ * inject one fault per lane. Lane l of word c of detector j (layout of tmcs_sample with
  * ceil(n_faults/64) words per detector) says whether fault first_fault+64c+l
  * flips detector j; observables likewise. first_fault must be a multiple of
  * 64. Errors: TMCS_E_INVALID (range), as tmcs_sample otherwise.
@@ -344,7 +346,9 @@ typedef struct {
  * operations thresholds and scaling", Methods "Simulation" and
  * "Statistics": each point needs enough shots to see logical errors) -- each
  * sampled as in tmcs_sample. This call samples such a set of jobs together.
- * Sample many circuits of uneven size on `stream`: the jobs share persistent
+ * Sample many circuits of uneven size on `stream`: the jobs share launches
+ * of the decoupled kernel (64 jobs each, CTAs dealt out by work), or, when one
+ * of them does not fit it or is denser in events than its arena, persistent
  * launches whose resident CTAs pull (job, tile) work items from a device
  * queue; a job that fills the GPU by itself (at least 16 chunks per SM) with
  * an event-signature program instead runs as its own tmcs_sample call, with

@@ -34,9 +34,9 @@
 //
 // Measured (one GB300, 2070 MHz; before = one lane per stream with refills,
 // 8-byte event slots per Pauli index): d=29 non-local CNOT, p = 1e-3, 2e6
-// shots (12.39 GB of output): 11.2 ms before, 9.2 ms now (1.34 TB/s); the
-// same at p = 1e-4: 6.6, 4.9 (2.5 TB/s); d=11, 1e7 shots: 3.28, 2.66; BB144
-// teleport, 3e6: 3.02, 2.06. What bounds it now is the appliers' chain: a
+// shots (12.39 GB of output): 11.2 ms before, 9.4 ms now (1.32 TB/s); the
+// same at p = 1e-4: 6.6, 4.9 (2.5 TB/s); d=11, 1e7 shots: 3.28, 2.61; BB144
+// teleport, 3e6: 3.02, 1.97. What bounds it now is the appliers' chain: a
 // step of d=29 costs them 6.6 k cycles of application, 4.2 k of flush and 1.1 k
 // of waiting.
 #include <cuda.h>  // CUtensorMap (encoded through the runtime's driver entry point)
@@ -276,10 +276,10 @@ struct FlowStepThread {
 // FAST: gap tables in shared memory, one table read per gap count, no
 // PAULI_CHANNEL_1 noise (a program without ebit decoherence, every p above
 // 2.1e-5); the other cases share the general kernel (tables through L1),
-// which counts gaps with one read in batches whose tables all allow it. Two kernels
-// instead of run-time branches: the walkers' code is about the size of the
-// instruction caches, and every branch not taken sits between the ones that
-// are (stalls without an instruction were 1.6 of 12.7 cycles per issue).
+// which counts gaps with one read in batches whose tables all allow it. Two
+// kernels instead of run-time branches: the walkers' code is about the size of
+// the instruction caches, and every branch not taken sits between the ones
+// that are (stalls without an instruction were 1.6 of 12.7 cycles per issue).
 // W: Philox calls of every stream's first window. One length per launch (the
 // best for the program's items together): kernels with all four lengths and a
 // choice per batch measured 320 against 310 ns per chunk on d=29, 2.78 against

@@ -2354,9 +2354,9 @@ static LaunchShape choose_shape_sig(const tmcs_circuit *c, uint64_t n_cols, cons
 // tiles one after another, so the time goes as tiles per CTA times a tile's
 // time, which measured as about one chunk's worth of fixed latency (the
 // steps' hand-overs) plus K chunks; K minimises that product. Measured
-// (best K / best time / time at the K chosen, us): d=29, 677 chunks 2 / 384
-// / 384; d=29, 150 chunks 1 / 126 / 126; d=11, 1563 chunks 4 / 74 / 74;
-// d=11, 157 chunks 2 / 44 / 45; BB144 teleport, 1563 chunks 4 / 141 / 156.
+// (best K / best time / time at the K chosen, us): d=29, 677 chunks 2 / 353
+// / 353; d=29, 150 chunks 1 / 97 / 97; d=11, 1563 chunks 4 / 50 / 50;
+// d=11, 157 chunks 2 / 22 / 24; BB144 teleport, 1563 chunks 4 / 92 / 92.
 // The ring is flow_shape_untimed's. A tile whose steps do not fit the arena
 // on any ring is not taken while a smaller one's do: at p = 1e-2 the product
 // rule alone took K = 8 for 1,216 chunks of d=11 (401 us, K = 2 254); one
